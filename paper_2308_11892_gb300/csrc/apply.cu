@@ -341,56 +341,110 @@ __global__ void k_identity(long long n, const double* __restrict__ vbase, T* __r
 // handles one row per 4-lane quad, lane r computing component r.  A row's
 // dependencies are read through their values, which start as a sentinel NaN:
 // a 4-vector that holds no sentinel is final.  Waits are bounded.
-template <class T>
-__device__ __forceinline__ bool wait_vec(const T* p, T* o, int* status, unsigned limit) {
-  for (unsigned s = 0;; ++s) {
-    ld_volatile4(p, o);
-    if (!is_sentinel(o[0]) && !is_sentinel(o[1]) && !is_sentinel(o[2]) && !is_sentinel(o[3]))
-      return true;
-    if (s + 1 >= limit) {  // `limit` polls saw the sentinel
-      dev_fail(status, DEV_TIMEOUT);
-      return false;
+// Rows are bound by memory latency, so every load that does not depend on
+// another row is issued before the first wait: dep_load reads the dependency
+// indices and factor rows of a batch of up to B dependencies, and dep_wait then
+// reads their y vectors together, so that a row whose dependencies are ready
+// costs one L2 round trip and not one for each of them; only the vectors that
+// still hold the sentinel are read again.  A vector found unwritten by `limit`
+// reads ends the wait (DEV_TIMEOUT).  S: stride between a lane's dependencies
+// (1: a quad takes all of them; 4: sixteen lanes share them).
+template <class T, int B, int S>
+struct Deps {
+  const T* yp[B];
+  T f[B][4], yv[B][4];
+  unsigned todo;
+};
+template <class T, int B, int S>
+__device__ __forceinline__ void dep_load(Deps<T, B, S>& D, int k, int ke,
+                                         const int32_t* __restrict__ ci,
+                                         const T* __restrict__ F, const T* y, int r) {
+  D.todo = 0;
+#pragma unroll
+  for (int q = 0; q < B; ++q)
+    if (k + S * q < ke) {
+      D.yp[q] = y + 4 * (size_t)ci[k + S * q];
+      ld4(F + 16 * (size_t)(k + S * q) + 4 * r, D.f[q]);
+      D.todo |= 1u << q;
     }
-    if ((s & 255u) == 255u && ld_volatile_i32(status) != DEV_OK) return false;
+}
+template <class T, int B, int S>
+__device__ __forceinline__ void dep_wait(Deps<T, B, S>& D, int* status, unsigned limit) {
+  for (unsigned s = 0; D.todo; ++s) {
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+      if (D.todo >> q & 1u) ld_volatile4(D.yp[q], D.yv[q]);
+#pragma unroll
+    for (int q = 0; q < B; ++q)
+      if ((D.todo >> q & 1u) && !is_sentinel(D.yv[q][0]) && !is_sentinel(D.yv[q][1]) &&
+          !is_sentinel(D.yv[q][2]) && !is_sentinel(D.yv[q][3]))
+        D.todo &= ~(1u << q);
+    if (!D.todo) return;
+    const bool out_of_polls = s + 1 >= limit;
+    if (out_of_polls) dev_fail(status, DEV_TIMEOUT);
+    if (out_of_polls || ((s & 255u) == 255u && ld_volatile_i32(status) != DEV_OK)) return;
   }
 }
 
 // acc minus, in the row's order, F_k y_{j_k} over its dependencies k in
-// [kb, ke), waiting for each y: the indices and factor blocks of the first
-// kPre dependencies are loaded before the first wait, so that when one
-// dependency arrives the next one's index and block are already in registers.
-template <class T>
+// [kb, ke), four lanes per row (lane r: component r).
+template <class T, int B>
 __device__ __forceinline__ T dep_chain(T acc, int kb, int ke, const int32_t* __restrict__ ci,
                                        const T* __restrict__ F, const T* y, int r, int* status,
-                                       unsigned lim) {
-  constexpr int kPre = 4;
-  int j[kPre];
-  T f[kPre][4];
-  const int np = ke - kb < kPre ? ke - kb : kPre;
+                                       unsigned limit) {
+  Deps<T, B, 1> D;
+  for (int k = kb; k < ke; k += B) {
+    dep_load(D, k, ke, ci, F, y, r);
+    dep_wait(D, status, limit);
+    // the products, then the subtractions, which alone chain in the fixed order
+    T d[B];
 #pragma unroll
-  for (int q = 0; q < kPre; ++q)
-    if (q < np) {
-      j[q] = ci[kb + q];
-      ld4(F + 16 * (size_t)(kb + q) + 4 * r, f[q]);
-    }
+    for (int q = 0; q < B; ++q)
+      if (k + q < ke) d[q] = dot4(D.f[q], D.yv[q]);
 #pragma unroll
-  for (int q = 0; q < kPre; ++q)
-    if (q < np) {
-      T yj[4];
-      wait_vec(y + 4 * (size_t)j[q], yj, status, lim);
-      acc = sub_rn(acc, dot4(f[q], yj));
-    }
-  for (int k = kb + kPre; k < ke; ++k) {
-    const int jj = ci[k];
-    T a[4], yj[4];
-    ld4(F + 16 * (size_t)k + 4 * r, a);
-    wait_vec(y + 4 * (size_t)jj, yj, status, lim);
-    acc = sub_rn(acc, dot4(a, yj));
+    for (int q = 0; q < B; ++q)
+      if (k + q < ke) acc = sub_rn(acc, d[q]);
   }
   return acc;
 }
 
-template <class T>
+// The same sum with sixteen lanes per row: lane 4 s + r takes the dependencies
+// s, s + 4, ... of a batch of 4 W and forms their products for component r, so
+// that a row's loads and products run side by side; every lane returns the sum.
+template <class T, int W>
+__device__ __forceinline__ T dep_chain16(T acc, int kb, int ke, const int32_t* __restrict__ ci,
+                                         const T* __restrict__ F, const T* y, int* status,
+                                         unsigned limit) {
+  const int lane = threadIdx.x & 31, slot = (lane >> 2) & 3, r = lane & 3, base = lane & 16;
+  const unsigned half = 0xffffu << base;
+  Deps<T, W, 4> D;
+  for (int k = kb; k < ke; k += 4 * W) {
+    dep_load(D, k + slot, ke, ci, F, y, r);
+    dep_wait(D, status, limit);
+    __syncwarp(half);
+    T d[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) d[w] = dot4(D.f[w], D.yv[w]);  // (unused past the row's end)
+#pragma unroll
+    for (int q = 0; q < 4 * W; ++q) {
+      const T v = __shfl_sync(half, d[q >> 2], base + 4 * (q & 3) + r);
+      if (k + q < ke) acc = sub_rn(acc, v);
+    }
+  }
+  return acc;
+}
+
+// The level-ordered solves: a warp claims the next group of 32 / LANES schedule
+// positions, LANES (4 or 16) lanes per row, B dependencies per lane and batch.
+// (Claiming the next group before the current one's wait measured 0-50% slower:
+// the claim's latency then delays the waits.)
+__device__ __forceinline__ unsigned claim_group(unsigned* ctr) {
+  unsigned g = 0;
+  if ((threadIdx.x & 31) == 0) g = atomicAdd(ctr, 1u);
+  return __shfl_sync(0xffffffffu, g, 0);
+}
+
+template <class T, int LANES, int B>
 __global__ void __launch_bounds__(256) k_ilu_fwd(int npos, const int32_t* __restrict__ ord,
                                                  const int32_t* __restrict__ Lrp,
                                                  const int32_t* __restrict__ Lci,
@@ -398,25 +452,24 @@ __global__ void __launch_bounds__(256) k_ilu_fwd(int npos, const int32_t* __rest
                                                  T* u, T* __restrict__ y2, Ctl* ctl,
                                                  const int* active) {
   if (!*active) return;
-  int lane = threadIdx.x & 31, sub = lane >> 2, r = lane & 3;
-  unsigned ngroups = (unsigned)((npos + 7) >> 3);
+  const int lane = threadIdx.x & 31, slot = (lane & (LANES - 1)) >> 2, r = lane & 3;
+  const unsigned ngroups = (unsigned)((npos + 32 / LANES - 1) / (32 / LANES));
   const unsigned lim = ctl->spin;
-  for (;;) {
-    unsigned gq = 0;
-    if (lane == 0) gq = atomicAdd(&ctl->fwd_ctr, 1u);
-    gq = __shfl_sync(0xffffffffu, gq, 0);
-    if (gq >= ngroups) return;
-    int pos = (int)(gq * 8 + sub);
-    int i = (pos < npos) ? ord[pos] : -1;
+  for (unsigned g; (g = claim_group(&ctl->fwd_ctr)) < ngroups;) {
+    const int pos = (int)(g * (32 / LANES)) + lane / LANES;
+    const int i = pos < npos ? ord[pos] : -1;
     if (i < 0) continue;
-    T acc = dep_chain<T>(r2[4 * (size_t)i + r], Lrp[pos], Lrp[pos + 1], Lci, Lv, u, r,
-                         &ctl->status, lim);
-    st_volatile(u + 4 * (size_t)i + r, desentinel(acc));
-    y2[4 * (size_t)i + r] = sentinel_of(T(0));
+    T acc = r2[4 * (size_t)i + r];
+    if (LANES == 4)
+      acc = dep_chain<T, B>(acc, Lrp[pos], Lrp[pos + 1], Lci, Lv, u, r, &ctl->status, lim);
+    else
+      acc = dep_chain16<T, B>(acc, Lrp[pos], Lrp[pos + 1], Lci, Lv, u, &ctl->status, lim);
+    if (slot == 0) st_volatile(u + 4 * (size_t)i + r, desentinel(acc));
+    if (slot == (LANES == 16 ? 1 : 0)) y2[4 * (size_t)i + r] = sentinel_of(T(0));
   }
 }
 
-template <class T>
+template <class T, int LANES, int B>
 __global__ void __launch_bounds__(256) k_ilu_bwd(int npos, const int32_t* __restrict__ ord,
                                                  const int32_t* __restrict__ Urp,
                                                  const int32_t* __restrict__ Uci,
@@ -427,41 +480,33 @@ __global__ void __launch_bounds__(256) k_ilu_bwd(int npos, const int32_t* __rest
                                                  T* __restrict__ zbase, const int* jptr,
                                                  size_t stride, Ctl* ctl, const int* active) {
   if (!*active) return;
-  int lane = threadIdx.x & 31, sub = lane >> 2, r = lane & 3;
-  unsigned ngroups = (unsigned)((npos + 7) >> 3);
+  const int lane = threadIdx.x & 31, slot = (lane & (LANES - 1)) >> 2, r = lane & 3;
+  const int base = lane & ~(LANES - 1);
+  const unsigned mask = (LANES == 16 ? 0xffffu : 0xfu) << base;
+  const unsigned ngroups = (unsigned)((npos + 32 / LANES - 1) / (32 / LANES));
   const unsigned lim = ctl->spin;
   T* z = zbase + (size_t)(*jptr) * stride;
-  for (;;) {
-    unsigned gq = 0;
-    if (lane == 0) gq = atomicAdd(&ctl->bwd_ctr, 1u);
-    gq = __shfl_sync(0xffffffffu, gq, 0);
-    if (gq >= ngroups) return;
-    int pos = (int)(gq * 8 + sub);
-    int i = (pos < npos) ? ord[pos] : -1;
+  for (unsigned g; (g = claim_group(&ctl->bwd_ctr)) < ngroups;) {
+    const int pos = (int)(g * (32 / LANES)) + lane / LANES;
+    const int i = pos < npos ? ord[pos] : -1;
     if (i < 0) continue;
-    // everything that does not depend on other rows is loaded before the
-    // dependency waits, so that only the waits and the arithmetic chain the
-    // levels (inv(U_ii) loaded after them cost one more memory latency per level)
-    T acc = u[4 * (size_t)i + r];
-    T d[4];
+    // inv(U_ii) and the first-stage part do not depend on other rows either
+    T acc = u[4 * (size_t)i + r], y1 = 0, d[4], s[4];
     ld4(Dinv + 16 * (size_t)pos + 4 * r, d);
-    T y1 = 0;
     if (zc) {
       const int ne = e1 < 0 ? 1 : 2;
       if (r == e0) y1 = zc[ne * (size_t)i];
       else if (r == e1) y1 = zc[ne * (size_t)i + 1];
     }
-    acc = dep_chain<T>(acc, Urp[pos], Urp[pos + 1], Uci, Uv, y2, r, &ctl->status, lim);
-    unsigned mask = 0xFu << (lane & ~3);
-    int q0 = lane & ~3;
-    T s0 = __shfl_sync(mask, acc, q0 + 0);
-    T s1 = __shfl_sync(mask, acc, q0 + 1);
-    T s2 = __shfl_sync(mask, acc, q0 + 2);
-    T s3 = __shfl_sync(mask, acc, q0 + 3);
-    T sv4[4] = {s0, s1, s2, s3};
-    T y = dot4(d, sv4);
-    st_volatile(y2 + 4 * (size_t)i + r, desentinel(y));
-    z[4 * (size_t)i + r] = y1 + y;
+    if (LANES == 4)
+      acc = dep_chain<T, B>(acc, Urp[pos], Urp[pos + 1], Uci, Uv, y2, r, &ctl->status, lim);
+    else
+      acc = dep_chain16<T, B>(acc, Urp[pos], Urp[pos + 1], Uci, Uv, y2, &ctl->status, lim);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] = __shfl_sync(mask, acc, base + q);
+    const T y = dot4(d, s);
+    if (slot == 0) st_volatile(y2 + 4 * (size_t)i + r, desentinel(y));
+    if (slot == (LANES == 16 ? 1 : 0)) z[4 * (size_t)i + r] = y1 + y;
   }
 }
 
@@ -611,24 +656,52 @@ void launch_vcycle(cptr_ctx* c, const T* b0, const int* active) {
   }
 }
 
+// One level-ordered solve with LANES lanes per row and B dependencies per lane.
+template <class T, int LANES, int B>
+void launch_levels_as(cptr_ctx* c, int grid, const T* zc, void* zbase, const int* jptr,
+                      size_t stride, const int* active, int which) {
+  cudaStream_t s = c->stream;
+  if (which != 2)
+    KL(c, k_ilu_fwd<T, LANES, B><<<grid, 256, 0, s>>>(c->npos_f, c->ord_f, c->Lrp, c->Lci,
+                                                      (const T*)c->Lv, (const T*)c->r2, (T*)c->u,
+                                                      (T*)c->y2, c->ctl, active));
+  if (which != 1)
+    KL(c, k_ilu_bwd<T, LANES, B><<<grid, 256, 0, s>>>(
+              c->npos_b, c->ord_b, c->Urp, c->Uci, (const T*)c->Uv, (const T*)c->Dinv,
+              (const T*)c->u, (T*)c->y2, zc, c->se0, c->se1, (T*)zbase, jptr, stride, c->ctl,
+              active));
+}
+
 template <class T>
 void launch_ilu_levels(cptr_ctx* c, const T* zc, void* zbase, const int* jptr, size_t stride,
                        const int* active, int which) {
-  cudaStream_t s = c->stream;
-  // warps claim groups of 8 rows in level order; the grid bounds how many rows
-  // are in flight (a few levels' worth: more only adds warps spinning on rows
-  // far ahead of the wavefront, whose polls compete for L2 with the solve)
-  // (measured on GB300: 3 blocks of 8 warps per SM beat 8 per SM by 3-8% on the
-  // 64x64x32, 1M-point kNN and 200x200x100 systems; fewer lose throughput)
-  int grid = c->lvl_grid_forced ? c->lvl_grid_forced : c->lvl_grid ? c->lvl_grid : c->nsm * 3;
-  if (which != 2)
-    KL(c, k_ilu_fwd<T><<<grid, 256, 0, s>>>(c->npos_f, c->ord_f, c->Lrp, c->Lci, (const T*)c->Lv,
-                                            (const T*)c->r2, (T*)c->u, (T*)c->y2, c->ctl, active));
-  if (which != 1)
-    KL(c, k_ilu_bwd<T><<<grid, 256, 0, s>>>(c->npos_b, c->ord_b, c->Urp, c->Uci, (const T*)c->Uv,
-                                            (const T*)c->Dinv, (const T*)c->u, (T*)c->y2, zc,
-                                            c->se0, c->se1, (T*)zbase, jptr, stride, c->ctl,
-                                            active));
+  // Warps claim groups of rows in level order; the grid (blocks of 8 warps per
+  // SM) bounds how many rows are in flight: more only adds warps polling L2 for
+  // rows far ahead of the wavefront, fewer lose throughput.
+  //
+  // Four lanes per row keep the most rows in flight, which wide levels need;
+  // sixteen shorten a row's chain when the levels are narrow (at most 32 rows
+  // per SM) and a row has many dependencies or FP64 products, whose issue rate
+  // binds the four-lane form.  Forward / backward in ms:
+  //   FP32, 1M-point cloud (570 rows per level, 5.2 dependencies): 16 lanes
+  //     1.85 / 1.98, 4 lanes 2.45 / 4.46 (one read after the other: 3.80 / 7.95);
+  //   FP32, 200x200x100 grid (8032 rows, 3): 4 lanes 0.73 / 0.80, 16 lanes
+  //     1.48 / 1.53 (0.93 / 1.02);
+  //   FP64, 110k-point cloud (179 rows): 16 lanes 0.88 / 1.33, 4 lanes
+  //     1.65 / 2.64 (1.94 / 3.88);
+  //   FP64, 150x110x57 grid (2986 rows): 0.53 / 0.63 against 0.61 / 0.70
+  //     (0.67 / 1.07); 200x200x100 grid: 1.66 / 1.93 against 1.14 / 1.32.
+  const bool f32 = sizeof(T) == 4;
+  const long long rows = c->nlev_f > 0 ? c->N / c->nlev_f : c->N;
+  const bool narrow = rows <= 32ll * c->nsm;
+  const bool long_rows = 2 * c->nnzL > 7ll * c->N;  // over 3.5 dependencies on average
+  const int forced = c->lvl_grid_forced;
+  if (narrow && (!f32 || long_rows))
+    launch_levels_as<T, 16, sizeof(T) == 4 ? 2 : 1>(c, forced ? forced : (f32 ? 2 : 3) * c->nsm,
+                                                    zc, zbase, jptr, stride, active, which);
+  else
+    launch_levels_as<T, 4, 3>(c, forced ? forced : (f32 ? 3 : 2) * c->nsm, zc, zbase, jptr,
+                              stride, active, which);
 }
 
 // which: 0 = forward and backward, 1 = forward only, 2 = backward only

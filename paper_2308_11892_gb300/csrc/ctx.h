@@ -299,9 +299,9 @@ struct cptr_ctx {
   // test hooks of the strip triangular solves: strips, solution-ring rows and
   // staging-ring bytes (CPTR_STRIP_P, CPTR_STRIP_RC, CPTR_STRIP_RING; 0 = automatic)
   int strip_p = 0, strip_rc = 0, strip_ring = 0;
-  // thread blocks of the level-scheduled triangular solves (0: chosen by the
-  // tuner; CPTR_LVL_GRID forces a value)
-  int lvl_grid = 0, lvl_grid_forced = 0;
+  // thread blocks of the level-scheduled triangular solves (0: by the rule of
+  // launch_ilu_levels; CPTR_LVL_GRID forces a value)
+  int lvl_grid_forced = 0;
   double phase_t0 = 0.0;
 };
 

@@ -118,6 +118,36 @@ __device__ __forceinline__ void ld4(const float* p, float* o) {
   o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
 }
 
+// N floats as doubles, on the integer pipes: a conversion instruction takes a
+// slot of the FP64 pipe like an FMA (also when it is predicated off), which
+// halves a kernel that converts every operand it multiplies.  Exact: a normal
+// float's bits are re-biased and zero keeps its sign; the rare others
+// (subnormal, infinite, NaN) are converted one by one in a loop, which the
+// compiler cannot turn into predicated instructions of the common path.
+template <int N>
+__device__ __forceinline__ void widen(const float* f, double* o) {
+  unsigned rare = 0;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const unsigned u = __float_as_uint(f[q]), m = u & 0x7fffffffu;
+    const unsigned hi = m ? (m >> 3) + 0x38000000u : 0u;
+    o[q] = __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+    if (m - 0x00800000u >= 0x7f000000u && m != 0u) rare |= 1u << q;
+  }
+  while (rare) {
+    const int k = __ffs(rare) - 1;
+    rare &= rare - 1;
+    float v = f[0];
+#pragma unroll
+    for (int q = 1; q < N; ++q)
+      if (q == k) v = f[q];
+    const double d = (double)v;
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (q == k) o[q] = d;
+  }
+}
+
 template <class T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

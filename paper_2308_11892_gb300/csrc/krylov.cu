@@ -19,6 +19,20 @@ inline int nblk(long long n, int per = kT) { return n > 0 ? ceil_div(n, per) : 1
 // ------------------------------------------------------------------ BSR SpMV
 // Four lanes per block row, lane r computing y_i[r]; each lane streams its
 // 32-byte row slice of every 128-byte block (the quad reads whole blocks).
+// Bound by FP64 issue: four FMAs per block and lane, and with x in FP32 as many
+// conversions again unless they run on the integer pipes (widen): 1.64 -> 0.81 ms
+// on the 200x200x100 grid (0.77 with x in FP64).
+__device__ __forceinline__ void ld4_wide(const double* p, double* o) { ld4(p, o); }
+__device__ __forceinline__ void ld4_wide(const float* p, double* o) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+  const float f[4] = {a.x, a.y, a.z, a.w};
+  widen<4>(f, o);
+}
+__device__ __forceinline__ void ld1_wide(const double* p, double* o) { *o = *p; }
+__device__ __forceinline__ void ld1_wide(const float* p, double* o) {
+  const float f = *p;
+  widen<1>(&f, o);
+}
 template <class TX>
 __global__ void __launch_bounds__(256) k_bsr_spmv(int N, const int32_t* __restrict__ rp,
                                                   const int32_t* __restrict__ ci,
@@ -40,7 +54,7 @@ __global__ void __launch_bounds__(256) k_bsr_spmv(int N, const int32_t* __restri
     double2 a01 = __ldg(reinterpret_cast<const double2*>(a));
     double2 a23 = __ldg(reinterpret_cast<const double2*>(a) + 1);
     double xj[4];
-    ld4(x + 4 * (size_t)j, xj);
+    ld4_wide(x + 4 * (size_t)j, xj);
     // one FMA chain: four FP64 operations per block and lane (the FP64 pipe,
     // not HBM, bounds this kernel on GB300)
     acc = fma(a01.x, xj[0], acc);
@@ -96,42 +110,73 @@ __device__ void combine_columns(const double* part, double* out, int nc) {
   }
 }
 
-// CGS2 pass 1: out[l] = V_l . w for l <= j.  Columns are taken eight at a time
-// so that every thread keeps eight independent loads in flight.
+// The CGS2 passes are bound by FP64 issue, and an FMA that is predicated off
+// takes its slot like any other: the columns are therefore cut into groups of
+// exactly the number there are (no padding), each a loop compiled for its size.
+
+// red[u * 8 + warp] = this warp's part of V_{l0+u} . w over the block's rows,
+// for G columns at once (G independent loads in flight per thread and row).
+template <int G>
+__device__ __forceinline__ void dot_group(Range R, long long n, const double* __restrict__ V,
+                                          const double* __restrict__ w, double* red) {
+  double acc[G];
+#pragma unroll
+  for (int u = 0; u < G; ++u) acc[u] = 0.0;
+#pragma unroll 2
+  for (long long i = R.lo + threadIdx.x; i < R.hi; i += blockDim.x) {
+    const double wi = w[i];
+#pragma unroll
+    for (int u = 0; u < G; ++u) acc[u] += V[(size_t)u * n + i] * wi;
+  }
+#pragma unroll
+  for (int u = 0; u < G; ++u) {
+    const double s = warp_sum(acc[u]);
+    if ((threadIdx.x & 31) == 0) red[u * 8 + (threadIdx.x >> 5)] = s;
+  }
+}
+
+// out[l] = V_l . w for the columns c0 <= l < nc, in near-equal groups of at most
+// eight; per-block partials, combined in block order by the last block.
+__device__ __forceinline__ void dot_columns(long long n, const double* __restrict__ V,
+                                            const double* __restrict__ w, int c0, int nc,
+                                            double* part, double* out, unsigned* ticket) {
+  __shared__ double red[64 * 8];
+  const Range R = block_range(n);
+  const int cols = nc - c0, groups = (cols + 7) / 8;
+  for (int g = 0, l = c0; g < groups; ++g) {
+    const int size = cols / groups + (g < cols % groups ? 1 : 0);
+    const double* Vl = V + (size_t)l * n;
+    double* rl = red + (size_t)(l - c0) * 8;
+    switch (size) {
+      case 1: dot_group<1>(R, n, Vl, w, rl); break;
+      case 2: dot_group<2>(R, n, Vl, w, rl); break;
+      case 3: dot_group<3>(R, n, Vl, w, rl); break;
+      case 4: dot_group<4>(R, n, Vl, w, rl); break;
+      case 5: dot_group<5>(R, n, Vl, w, rl); break;
+      case 6: dot_group<6>(R, n, Vl, w, rl); break;
+      case 7: dot_group<7>(R, n, Vl, w, rl); break;
+      default: dot_group<8>(R, n, Vl, w, rl); break;
+    }
+    l += size;
+  }
+  __syncthreads();
+  for (int l = c0 + (int)threadIdx.x; l < nc; l += blockDim.x) {
+    double s = 0.0;
+    for (int q = 0; q < 8; ++q) s += red[(l - c0) * 8 + q];
+    part[(size_t)l * gridDim.x + blockIdx.x] = s;
+  }
+  if (last_block_ticket(ticket)) {
+    combine_columns(part + (size_t)c0 * gridDim.x, out + c0, cols);
+    if (threadIdx.x == 0) *ticket = 0u;
+  }
+}
+
+// CGS2 pass 1: out[l] = V_l . w for l <= j.
 __global__ void __launch_bounds__(256) k_cgs_dot(long long n, const double* __restrict__ V,
                                                  const double* __restrict__ w, double* part,
                                                  double* out, Ctl* ctl) {
   if (!ctl->active) return;
-  __shared__ double red[64 * 8];
-  int nc = ctl->j + 1;
-  Range R = block_range(n);
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int lg = 0; lg < nc; lg += 8) {
-    double acc[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc[u] = 0.0;
-    for (long long i = R.lo + threadIdx.x; i < R.hi; i += blockDim.x) {
-      double wi = w[i];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (lg + u < nc) acc[u] += V[(size_t)(lg + u) * n + i] * wi;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      double s = warp_sum(acc[u]);
-      if (lane == 0 && lg + u < nc) red[(lg + u) * 8 + warp] = s;
-    }
-  }
-  __syncthreads();
-  for (int l = threadIdx.x; l < nc; l += blockDim.x) {
-    double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += red[l * 8 + q];
-    part[(size_t)l * gridDim.x + blockIdx.x] = s;
-  }
-  if (last_block_ticket(&ctl->red_ctr[0])) {
-    combine_columns(part, out, nc);
-    if (threadIdx.x == 0) ctl->red_ctr[0] = 0u;
-  }
+  dot_columns(n, V, w, 0, ctl->j + 1, part, out, &ctl->red_ctr[0]);
 }
 
 // CGS2 pass 2: w -= V h1, then out[l] = V_l . w, with the dot accumulators
@@ -139,7 +184,43 @@ __global__ void __launch_bounds__(256) k_cgs_dot(long long n, const double* __re
 // read of V_l[i] comes from L1, and the block needs no shared-memory tile
 // (several blocks per SM).  The update uses all (at most MAXH) columns; the
 // dots are formed here for the first MAXC of them (the rest, if any, by
-// k_cgs_dot_from on the updated w).
+// k_cgs_dot_from on the updated w).  upd_dot_rows is compiled for every
+// number of dots: 1.44 -> 0.53 ms on average over an FGMRES(50) solve of 19
+// iterations on the 200x200x100 grid (all 32 accumulators issued before), and
+// k_cgs_dot 0.41 -> 0.31 ms (groups of eight before).
+template <int NC>
+__device__ __forceinline__ void upd_dot_rows(Range R, long long n, int nh,
+                                             const double* __restrict__ V,
+                                             double* __restrict__ w, const double* hs,
+                                             double* red) {
+  double acc[NC];
+#pragma unroll
+  for (int l = 0; l < NC; ++l) acc[l] = 0.0;
+  for (long long i = R.lo + threadIdx.x; i < R.hi; i += blockDim.x) {
+    double wi = w[i];
+#pragma unroll 8
+    for (int l = 0; l < nh; ++l) wi -= hs[l] * V[(size_t)l * n + i];
+    w[i] = wi;
+#pragma unroll
+    for (int l = 0; l < NC; ++l) acc[l] += V[(size_t)l * n + i] * wi;
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int l = 0; l < NC; ++l) {
+    const double s = warp_sum(acc[l]);
+    if (lane == 0) red[l * 8 + warp] = s;
+  }
+}
+template <int NC, int MAXC>
+__device__ __forceinline__ void upd_dot_pick(Range R, long long n, int nh, int nc,
+                                             const double* __restrict__ V,
+                                             double* __restrict__ w, const double* hs,
+                                             double* red) {
+  if constexpr (NC < MAXC) {
+    if (nc > NC) return upd_dot_pick<NC + 1, MAXC>(R, n, nh, nc, V, w, hs, red);
+  }
+  upd_dot_rows<NC>(R, n, nh, V, w, hs, red);
+}
 template <int MAXC, int MAXH>
 __global__ void __launch_bounds__(256) k_cgs_upd_dot_reg(long long n,
                                                          const double* __restrict__ V,
@@ -152,27 +233,8 @@ __global__ void __launch_bounds__(256) k_cgs_upd_dot_reg(long long n,
   const int nh = ctl->j + 1;
   const int nc = nh < MAXC ? nh : MAXC;
   for (int l = threadIdx.x; l < nh; l += blockDim.x) hs[l] = h1[l];
-  double acc[MAXC];
-#pragma unroll
-  for (int l = 0; l < MAXC; ++l) acc[l] = 0.0;
   __syncthreads();
-  Range R = block_range(n);
-  for (long long i = R.lo + threadIdx.x; i < R.hi; i += blockDim.x) {
-    double wi = w[i];
-#pragma unroll 8
-    for (int l = 0; l < nh; ++l) wi -= hs[l] * V[(size_t)l * n + i];
-    w[i] = wi;
-#pragma unroll
-    for (int l = 0; l < MAXC; ++l)
-      if (l < nc) acc[l] += V[(size_t)l * n + i] * wi;
-  }
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-  for (int l = 0; l < MAXC; ++l) {
-    if (l >= nc) break;
-    double s = warp_sum(acc[l]);
-    if (lane == 0) red[l * 8 + warp] = s;
-  }
+  upd_dot_pick<1, MAXC>(block_range(n), n, nh, nc, V, w, hs, red);
   __syncthreads();
   for (int l = threadIdx.x; l < nc; l += blockDim.x) {
     double s = 0.0;
@@ -186,43 +248,12 @@ __global__ void __launch_bounds__(256) k_cgs_upd_dot_reg(long long n,
 }
 
 // out[l] = V_l . w for the columns c0 <= l <= j (nothing when j < c0): the
-// second-pass dots beyond the register kernel's first MAXC columns, in
-// k_cgs_dot's arrangement (eight columns at a time, fixed reduction order).
+// second-pass dots beyond the register kernel's first MAXC columns.
 __global__ void __launch_bounds__(256) k_cgs_dot_from(long long n, const double* __restrict__ V,
                                                       const double* __restrict__ w, int c0,
                                                       double* part, double* out, Ctl* ctl) {
-  if (!ctl->active) return;
-  const int nc = ctl->j + 1;
-  if (nc <= c0) return;
-  __shared__ double red[64 * 8];
-  Range R = block_range(n);
-  int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int lg = c0; lg < nc; lg += 8) {
-    double acc[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) acc[u] = 0.0;
-    for (long long i = R.lo + threadIdx.x; i < R.hi; i += blockDim.x) {
-      double wi = w[i];
-#pragma unroll
-      for (int u = 0; u < 8; ++u)
-        if (lg + u < nc) acc[u] += V[(size_t)(lg + u) * n + i] * wi;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      double s = warp_sum(acc[u]);
-      if (lane == 0 && lg + u < nc) red[(lg + u - c0) * 8 + warp] = s;
-    }
-  }
-  __syncthreads();
-  for (int l = c0 + (int)threadIdx.x; l < nc; l += blockDim.x) {
-    double s = 0.0;
-    for (int q = 0; q < 8; ++q) s += red[(l - c0) * 8 + q];
-    part[(size_t)l * gridDim.x + blockIdx.x] = s;
-  }
-  if (last_block_ticket(&ctl->red_ctr[0])) {
-    combine_columns(part + (size_t)c0 * gridDim.x, out + c0, nc - c0);
-    if (threadIdx.x == 0) ctl->red_ctr[0] = 0u;
-  }
+  if (!ctl->active || ctl->j < c0) return;
+  dot_columns(n, V, w, c0, ctl->j + 1, part, out, &ctl->red_ctr[0]);
 }
 
 // CGS2 pass 3: w -= V h2 and ||w||^2; the last block forms column j of the
@@ -384,7 +415,12 @@ __global__ void k_xupdate(long long n, double* __restrict__ x, const TZ* __restr
   long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   double xi = x[i];
-  for (int l = 0; l < k; ++l) xi += ys[l] * (double)Z[(size_t)l * n + i];
+#pragma unroll 4
+  for (int l = 0; l < k; ++l) {
+    double z;
+    ld1_wide(Z + (size_t)l * n + i, &z);
+    xi += ys[l] * z;
+  }
   x[i] = xi;
 }
 

@@ -293,7 +293,8 @@ struct cptr_ctx {
   double phase_ms[CPTR_PHASE_COUNT] = {};  // per phase, last cptr_setup
   bool force_fallback = false;  // CPTR_SETUP_FALLBACK=1: thread-per-row setup kernels only
   // test hooks: one SpGEMM path for every row (CPTR_SPGEMM_PATH: 1 ordered-table
-  // block kernel, 2 bucketed block kernel, 3 global-scratch kernel) and one
+  // block kernel, 2 bucketed block kernel, 3 global-scratch kernel, 4/5/6 every row
+  // starts in the smallest, the 512-column and the block-wide class) and one
   // ext+i path (CPTR_INTERP_PATH: 1 wide blocks, 2 global-scratch kernel)
   int spgemm_path = 0, interp_path = 0;
   // test hooks of the strip triangular solves: strips, solution-ring rows and

@@ -787,105 +787,6 @@ __global__ void k_spgemm_deferred(int n, const int32_t* __restrict__ cnt,
   bytes[k] = (long long)((spgemm_smem(hs, na < 1 ? 1 : na) + 255) & ~(size_t)255);
 }
 
-// Rows of C = A B with at most kSpwProd products, one warp per row: the
-// products are staged in shared memory, ranked by (column, product index) and
-// each output column is summed by one lane over its products in that order,
-// i.e. in the order of the entries of A, starting from 0.0 (the same sums as
-// k_spgemm_row).  Other rows are appended to rows[] for the block kernel.
-constexpr int kSpwProd = 64;
-constexpr int kSpwWarps = 8;
-struct SpwSmem {
-  int soff[kSpwProd + 1];  // first product of each A entry
-  int bst[kSpwProd];       // start of each A entry's B row
-  double sa[kSpwProd];     // A values
-  int key[kSpwProd];       // product columns, then sorted columns
-  int skey[kSpwProd];
-  double val[kSpwProd];    // products, then in sorted order
-  double sval[kSpwProd];
-};
-__global__ void __launch_bounds__(32 * kSpwWarps) k_spgemm_warp(
-    int n, const int32_t* __restrict__ arp, const int32_t* __restrict__ aci,
-    const double* __restrict__ av, const int32_t* __restrict__ brp,
-    const int32_t* __restrict__ bci, const double* __restrict__ bv,
-    const int32_t* __restrict__ prods, const long long* __restrict__ toff,
-    int32_t* __restrict__ cci, double* __restrict__ cv, int32_t* __restrict__ cnt,
-    int32_t* __restrict__ rows, int* nrows) {
-  __shared__ SpwSmem sm_all[kSpwWarps];
-  const int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (i >= n) return;
-  SpwSmem& W = sm_all[threadIdx.x >> 5];
-  const int t0 = arp[i], nA = arp[i + 1] - t0, T = prods[i];
-  if (T > kSpwProd || nA > kSpwProd) {
-    if (lane == 0) rows[atomicAdd(nrows, 1)] = i;
-    return;
-  }
-  // A entries: B-row starts and lengths, offsets by an inclusive warp scan
-  int carry = 0;
-  if (lane == 0) W.soff[0] = 0;
-  for (int e0 = 0; e0 < nA; e0 += 32) {
-    const int e = e0 + lane;
-    int len = 0;
-    if (e < nA) {
-      const int k = aci[t0 + e];
-      const int b = brp[k];
-      len = brp[k + 1] - b;
-      W.bst[e] = b;
-      W.sa[e] = av[t0 + e];
-    }
-    int x = len;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
-    }
-    if (e < nA) W.soff[e + 1] = carry + x;
-    carry += __shfl_sync(0xffffffffu, x, 31);
-  }
-  __syncwarp();
-  // products: column and value a_ik b_kj
-  for (int p = lane; p < T; p += 32) {
-    int lo = 0, hi = nA - 1;  // entry e with soff[e] <= p < soff[e+1]
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (W.soff[mid] <= p) lo = mid; else hi = mid - 1;
-    }
-    const int src = W.bst[lo] + (p - W.soff[lo]);
-    W.key[p] = bci[src];
-    W.val[p] = W.sa[lo] * bv[src];
-  }
-  __syncwarp();
-  // rank by (column, product index)
-  for (int p = lane; p < T; p += 32) {
-    const int k = W.key[p];
-    int r = 0;
-    for (int q = 0; q < T; ++q) {
-      const int kq = W.key[q];
-      r += kq < k || (kq == k && q < p);
-    }
-    W.skey[r] = k;
-    W.sval[r] = W.val[p];
-  }
-  __syncwarp();
-  // one lane per distinct column sums its run
-  int u = 0;
-  const long long o = toff[i];
-  for (int r0 = 0; r0 < T; r0 += 32) {
-    const int r = r0 + lane;
-    const bool head = r < T && (r == 0 || W.skey[r] != W.skey[r - 1]);
-    const unsigned hb = __ballot_sync(0xffffffffu, head);
-    if (head) {
-      const int col = W.skey[r];
-      double sum = 0.0;
-      for (int q = r; q < T && W.skey[q] == col; ++q) sum += W.sval[q];
-      const int qo = u + __popc(hb & ((1u << lane) - 1u));
-      cci[o + qo] = col;
-      cv[o + qo] = sum;
-    }
-    u += __popc(hb);
-  }
-  if (lane == 0) cnt[i] = u;
-}
-
 // Rows of C = A B with at most tprod products, one block per row (rows[] when
 // given).  Every product is formed once; the distinct columns are collected
 // in a hash set and sorted; the products are bucketed by output column in
@@ -2238,6 +2139,62 @@ __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int 
 
 inline int nblk(long long n) { return n > 0 ? ceil_div(n, kT) : 1; }
 
+#include "spgemm_acc.cuh"
+
+// Stream-ordered scratch of one setup step, given back when the step ends.
+struct Scratch {
+  cptr_ctx* c;
+  std::vector<void*> p;
+  explicit Scratch(cptr_ctx* ctx) : c(ctx) {}
+  Scratch(const Scratch&) = delete;
+  ~Scratch() {
+    for (void* q : p) cudaFreeAsync(q, c->stream);
+  }
+  template <class T>
+  T* get(size_t count) {
+    void* q = nullptr;
+    if (cudaMallocAsync(&q, sizeof(T) * count + 16, c->stream) != cudaSuccess) {
+      cudaGetLastError();
+      ctx_set_err(c, "device allocation of setup scratch failed");
+      return nullptr;
+    }
+    p.push_back(q);
+    return (T*)q;
+  }
+};
+
+template <int H>
+cptr_status acc_launch(cptr_ctx* c, void (*kern)(AccArgs, int, int), int rows_per_block, int rows,
+                       AccArgs a, int cls, int from) {
+  const size_t smem = acc_table_bytes<H>() * rows_per_block;
+  if (smem > 48 * 1024) CTX_CUDA(c, raise_smem_limit(c, (const void*)kern));
+  const int blocks = std::min(ceil_div(rows, rows_per_block), 1 << 20);
+  KL(c, kern<<<blocks, kAccThreads, smem, c->stream>>>(a, cls, from));
+  return CPTR_OK;
+}
+// Rows [from, ...) of class cls (about `rows` of them) with the class's kernel.
+// Short rows of B (at most six entries on average: interpolation operators) take
+// the lane-group kernels up to 256 columns, others a warp per row.
+cptr_status acc_run(cptr_ctx* c, AccArgs a, int cls, int from, int rows, bool short_b) {
+  constexpr int W = kAccThreads / 32;
+  switch (cls) {
+    case 0:
+      return short_b ? acc_launch<64>(c, k_acc_group<4, 64>, 8 * W, rows, a, cls, from)
+                     : acc_launch<64>(c, k_acc_flat<64>, W, rows, a, cls, from);
+    case 1: return acc_launch<128>(c, k_acc_flat<128>, W, rows, a, cls, from);
+    case 2: return acc_launch<256>(c, k_acc_flat<256>, W, rows, a, cls, from);
+    case 3: return acc_launch<512>(c, k_acc_flat<512>, W, rows, a, cls, from);
+    case 4: return acc_launch<1024>(c, k_acc_flat<1024>, W, rows, a, cls, from);
+    case 5: return acc_launch<2048>(c, k_acc_flat<2048>, W, rows, a, cls, from);
+    default: {
+      CTX_CUDA(c, raise_smem_limit(c, (const void*)k_acc_big));
+      KL(c, k_acc_big<<<std::min(rows, 1 << 16), 32 * kBigWarps, (size_t)kBigCols * 16,
+                        c->stream>>>(a, from));
+      return CPTR_OK;
+    }
+  }
+}
+
 // A product's distinct column count is at most its product count `bound`;
 // where that passes 2^31 - 1 the 32-bit row pointers could wrap, so the exact
 // count is taken in 64 bits first and a total past the limit is refused (the
@@ -2260,102 +2217,126 @@ cptr_status check_count_fits(cptr_ctx* c, const int32_t* cnt, int n, long long b
 // tables fit in kCap slots.
 cptr_status spgemm_fallback(cptr_ctx* c, const DCSR& A, const DCSR& B, DCSR& C);
 
-// C = A * B: block-per-row symbolic count, row pointers, block-per-row fill;
-// falls back to the batched thread-per-row hash kernel when a row's column
-// set does not fit in shared memory.
+// Rows up to which a product is one launch: every warp of the GPU has one or two.
+constexpr int kAccOneClass = 4096;
+
+// C = A * B in one pass: every row writes its sorted columns and sums into a slot
+// as long as its product count (the accumulators of spgemm_acc.cuh; rows too wide
+// for them take k_spgemm_row with tables in global scratch), then the rows are
+// compacted behind the row pointers.
 cptr_status spgemm(cptr_ctx* c, const DCSR& A, const DCSR& B, DCSR& C) {
   if (c->force_fallback) return spgemm_fallback(c, A, B, C);
-  int n = A.n;
-  int32_t *hs, *cnt;
-  int* flags;
-  int32_t* prods;
-  CTX_ALLOC(c, hs, int32_t, n + 1, true);
-  CTX_ALLOC(c, cnt, int32_t, n + 1, true);
-  CTX_ALLOC(c, prods, int32_t, n + 1, true);
-  CTX_ALLOC(c, flags, int, 8, true);
-  CTX_CUDA(c, cudaMemsetAsync(flags, 0, 8 * sizeof(int), c->stream));
+  const int n = A.n;
+  const bool acc = c->spgemm_path == 0 || c->spgemm_path > 3;
+  Scratch scr(c);
+  int32_t* hs = scr.get<int32_t>(n + 1);
+  int32_t* cnt = scr.get<int32_t>(n + 1);
+  int32_t* prods = scr.get<int32_t>(n + 1);
+  int* flags = scr.get<int>(8 + kAccClasses + 1);
+  long long* toff = scr.get<long long>(n + 1);
+  int32_t* lists = acc ? scr.get<int32_t>((size_t)(kAccClasses + 1) * n) : nullptr;
+  if (!hs || !cnt || !prods || !flags || !toff || (acc && !lists)) return CPTR_ERR_NOMEM;
+  CTX_CUDA(c, cudaMemsetAsync(flags, 0, (8 + kAccClasses + 1) * sizeof(int), c->stream));
   KL(c, k_spgemm_ub<<<nblk(n), kT, 0, c->stream>>>(n, A.rp, A.ci, B.rp, hs, prods, B.m,
                                                     flags + 4));
   cptr_status st;
-  // product offsets; the maxima and the product total come back in one read
-  long long* toff;
-  CTX_ALLOC(c, toff, long long, n + 1, true);
+  // product offsets; the maxima, class sizes and product total in one read
   st = scan_i64(c, prods, toff, n, nullptr);
   if (st) return st;
+  AccArgs args{n,   A.rp,    A.ci,    A.v, B.rp,  B.ci,      B.v,
+               toff, nullptr, nullptr, cnt, lists, flags + 8, -1};
+  // a few thousand rows are one launch whatever their class: no binning, the
+  // class of the longest row for all of them
+  const bool one_class = acc && c->spgemm_path == 0 && n <= kAccOneClass;
+  if (acc && !one_class) {
+    // test hooks: 4 starts every row in the smallest class, 5 in the one of 512
+    // columns, 6 in the last
+    const int path = c->spgemm_path;
+    KL(c, k_acc_bin<<<nblk(n), kT, 0, c->stream>>>(args, prods,
+                                                    path == 4 ? 0 : path == 5 ? 3
+                                                    : path == 6 ? kAccBig : -1));
+  }
   struct {
-    int mx3[3];
-    int pad;
+    int mx3[4];
+    int ncls[kAccClasses + 1];
     long long nprod;
   } hv;
-  CTX_CUDA(c, cudaMemcpyAsync(hv.mx3, flags + 4, 3 * sizeof(int), cudaMemcpyDeviceToHost,
-                              c->stream));
+  CTX_CUDA(c, cudaMemcpyAsync(hv.mx3, flags + 4, (4 + kAccClasses + 1) * sizeof(int),
+                              cudaMemcpyDeviceToHost, c->stream));
   CTX_CUDA(c, cudaMemcpyAsync(&hv.nprod, toff + n, sizeof(long long), cudaMemcpyDeviceToHost,
                               c->stream));
   CTX_CUDA(c, cudaStreamSynchronize(c->stream));
   const int* mx3 = hv.mx3;
   const long long nprod = hv.nprod;
-  const int kSmemHs = 4096, kSmemRow = 1024, kSmemProd = 1024;  // shared-memory pass limits
-  const int mx = mx3[0];
-  int hsz = mx < 64 ? 64 : (mx > kSmemHs ? kSmemHs : mx);
-  int thr = hsz >= 2048 ? 256 : 128;
-  int tprod = 64;
-  while (tprod < mx3[1] && tprod < kSmemProd) tprod <<= 1;
-  int maxa = mx3[2] < 1 ? 1 : (mx3[2] > kSmemRow ? kSmemRow : mx3[2]);
-  const size_t ssm = sps_layout(hsz, tprod, maxa).total;
-  // one pass: every row writes its sorted columns into a slot as long as its
-  // product count, then the rows are compacted behind the row pointers
-  int32_t* tci;
-  double* tv;
-  CTX_ALLOC(c, tci, int32_t, nprod + 1, true);
-  CTX_ALLOC(c, tv, double, nprod + 1, true);
-  // rows with few products: one warp per row, the others one block per row
-  // (the warp pass runs when the average row has at most kSpwProd products);
-  // rows too large for shared memory are deferred (flags[0] counts them)
-  // Bucketing pays where the ordered-product table wastes the most: long A
-  // rows (the table's column sums scan every A entry) or few products per
-  // row; short A rows with many products (R (AP) on coarse levels) keep the
-  // table kernel, whose shared memory does not grow with the product count.
-  const bool bucketed = c->spgemm_path == 2 ||
-                        (c->spgemm_path == 0 && (A.nnz >= 16ll * n || nprod <= 256ll * n));
-  size_t tsm = 0;
-  if (!bucketed) {
-    tsm = spgemm_smem(hsz, maxa);
-    CTX_CUDA(c, cudaFuncSetAttribute(k_spgemm_row<false>,
-                                     cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-  }
-  int32_t* brows = nullptr;
-  int nb = c->spgemm_path == 3 ? 0 : n;
-  if (c->spgemm_path == 3) {  // every row to the global-scratch pass
+  int32_t* tci = scr.get<int32_t>(nprod + 1);
+  double* tv = scr.get<double>(nprod + 1);
+  if (!tci || !tv) return CPTR_ERR_NOMEM;
+  int ndef = 0;  // rows left for the global-scratch kernel (cnt = -1)
+  if (acc) {
+    args.cci = tci;
+    args.cv = tv;
+    const bool short_b = B.nnz <= 6ll * B.n;
+    int done[kAccClasses] = {};
+    if (one_class) {
+      args.all = acc_class(mx3[1]);
+      st = acc_run(c, args, args.all, 0, n, false);
+      if (st) return st;
+      CTX_CUDA(c, cudaMemcpyAsync(hv.ncls, flags + 8, sizeof(hv.ncls), cudaMemcpyDeviceToHost,
+                                  c->stream));
+      CTX_CUDA(c, cudaStreamSynchronize(c->stream));
+    }
+    for (;;) {  // a class launched after a smaller one also takes the rows it deferred
+      bool left = false;
+      for (int k = 0; k < kAccClasses; ++k) {
+        if (hv.ncls[k] <= done[k]) continue;
+        left = true;
+        st = acc_run(c, args, k, done[k], hv.ncls[k] - done[k], short_b);
+        if (st) return st;
+        done[k] = -1;  // launched: done up to the count read below
+      }
+      if (!left) break;
+      CTX_CUDA(c, cudaMemcpyAsync(hv.ncls, flags + 8, sizeof(hv.ncls), cudaMemcpyDeviceToHost,
+                                  c->stream));
+      CTX_CUDA(c, cudaStreamSynchronize(c->stream));
+      for (int k = 0; k < kAccClasses; ++k)
+        if (done[k] < 0) done[k] = hv.ncls[k];
+    }
+    ndef = hv.ncls[kAccClasses];
+  } else if (c->spgemm_path == 3) {  // every row to the global-scratch pass
     CTX_CUDA(c, cudaMemsetAsync(cnt, 0xff, sizeof(int32_t) * n, c->stream));
-    CTX_CUDA(c, cudaMemcpyAsync(flags, &n, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-  } else if (c->spgemm_path == 0 && nprod <= (long long)kSpwProd * n) {
-    CTX_ALLOC(c, brows, int32_t, n + 1, true);
-    KL(c, k_spgemm_warp<<<nblk((long long)n * 32), 32 * kSpwWarps, 0, c->stream>>>(
-              n, A.rp, A.ci, A.v, B.rp, B.ci, B.v, prods, toff, tci, tv, cnt, brows, flags + 3));
-    CTX_CUDA(c, cudaMemcpyAsync(&nb, flags + 3, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    ndef = n;
+  } else {
+    // test hooks: the block kernels for every row that fits (1 ordered-table,
+    // 2 bucketed); flags[0] counts the rows they defer
+    const int kSmemHs = 4096, kSmemRow = 1024, kSmemProd = 1024;
+    const int mx = mx3[0];
+    const int hsz = mx < 64 ? 64 : (mx > kSmemHs ? kSmemHs : mx);
+    const int thr = hsz >= 2048 ? 256 : 128;
+    int tprod = 64;
+    while (tprod < mx3[1] && tprod < kSmemProd) tprod <<= 1;
+    const int maxa = mx3[2] < 1 ? 1 : (mx3[2] > kSmemRow ? kSmemRow : mx3[2]);
+    if (c->spgemm_path == 2) {
+      CTX_CUDA(c, raise_smem_limit(c, (const void*)k_spgemm_sorted));
+      KL(c, k_spgemm_sorted<<<n, thr, sps_layout(hsz, tprod, maxa).total, c->stream>>>(
+                hsz, tprod, maxa, hs, A.rp, A.ci, A.v, B.rp, B.ci, B.v, prods, toff, tci, tv, cnt,
+                flags, nullptr));
+    } else {
+      CTX_CUDA(c, cudaFuncSetAttribute(k_spgemm_row<false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+      KL(c, k_spgemm_row<false><<<n, thr, spgemm_smem(hsz, maxa), c->stream>>>(
+                hsz, maxa, hs, A.rp, A.ci, A.v, B.rp, B.ci, B.v, toff, tci, tv, cnt, flags,
+                nullptr, nullptr, nullptr));
+    }
+    CTX_CUDA(c, cudaMemcpyAsync(&ndef, flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     CTX_CUDA(c, cudaStreamSynchronize(c->stream));
   }
-  if (bucketed)
-    CTX_CUDA(c, raise_smem_limit(c, (const void*)k_spgemm_sorted));
-  if (nb > 0 && bucketed)
-    KL(c, k_spgemm_sorted<<<nb, thr, ssm, c->stream>>>(hsz, tprod, maxa, hs, A.rp, A.ci, A.v,
-                                                       B.rp, B.ci, B.v, prods, toff, tci, tv, cnt,
-                                                       flags, brows));
-  else if (nb > 0)
-    KL(c, k_spgemm_row<false><<<nb, thr, tsm, c->stream>>>(hsz, maxa, hs, A.rp, A.ci, A.v, B.rp,
-                                                            B.ci, B.v, toff, tci, tv, cnt, flags,
-                                                            brows, nullptr, nullptr));
-  int ndef = 0;
-  CTX_CUDA(c, cudaMemcpyAsync(&ndef, flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-  CTX_CUDA(c, cudaStreamSynchronize(c->stream));
   if (ndef > 0) {
     // rows too wide for shared memory: the same algorithm, tables in global scratch
-    int32_t *rows, *rbytes;
-    long long *goff, *rb64;
-    CTX_ALLOC(c, rows, int32_t, ndef + 1, true);
-    CTX_ALLOC(c, rb64, long long, ndef + 1, true);
-    CTX_ALLOC(c, rbytes, int32_t, ndef + 1, true);
-    CTX_ALLOC(c, goff, long long, ndef + 1, true);
+    int32_t* rows = scr.get<int32_t>(ndef + 1);
+    int32_t* rbytes = scr.get<int32_t>(ndef + 1);
+    long long* rb64 = scr.get<long long>(ndef + 1);
+    long long* goff = scr.get<long long>(ndef + 1);
+    if (!rows || !rbytes || !rb64 || !goff) return CPTR_ERR_NOMEM;
     CTX_CUDA(c, cudaMemsetAsync(flags + 2, 0, sizeof(int), c->stream));
     KL(c, k_spgemm_deferred<<<nblk(n), kT, 0, c->stream>>>(n, cnt, A.rp, hs, rows, rb64,
                                                             flags + 2));
@@ -2363,7 +2344,7 @@ cptr_status spgemm(cptr_ctx* c, const DCSR& A, const DCSR& B, DCSR& C) {
     long long gtot = 0;
     st = scan_i64(c, rbytes, goff, ndef, &gtot);
     if (st) return st;
-    unsigned char* gscr = (unsigned char*)ctx_alloc(c, (size_t)gtot + 256, true);
+    unsigned char* gscr = scr.get<unsigned char>((size_t)gtot + 256);
     if (!gscr) return CPTR_ERR_NOMEM;
     CTX_CUDA(c, cudaMemsetAsync(flags + 1, 0, sizeof(int), c->stream));
     KL(c, k_spgemm_row<true><<<ndef, 256, 0, c->stream>>>(0, 0, hs, A.rp, A.ci, A.v, B.rp, B.ci,

@@ -295,7 +295,8 @@ struct cptr_ctx {
   // test hooks: one SpGEMM path for every row (CPTR_SPGEMM_PATH: 1 ordered-table
   // block kernel, 2 bucketed block kernel, 3 global-scratch kernel, 4/5/6 every row
   // starts in the smallest, the 512-column and the block-wide class) and one
-  // ext+i path (CPTR_INTERP_PATH: 1 wide blocks, 2 global-scratch kernel)
+  // ext+i path (CPTR_INTERP_PATH: 1 wide blocks, 2 global-scratch kernel, 3/4/5 every F
+  // point starts in class 0/1/2 of the lane-group kernels)
   int spgemm_path = 0, interp_path = 0;
   // test hooks of the strip triangular solves: strips, solution-ring rows and
   // staging-ring bytes (CPTR_STRIP_P, CPTR_STRIP_RC, CPTR_STRIP_RING; 0 = automatic)

@@ -1169,24 +1169,32 @@ __host__ __device__ inline InterpSmem interp_layout(int hs, int rl, int kcap, in
   L.total = o;
   return L;
 }
-enum { IF_S = 1, IF_SAME = 2, IF_C = 4, IF_DIAG = 8 };
+enum { IF_S = 1, IF_SAME = 2, IF_C = 4, IF_DIAG = 8, IF_NEG = 16 };
 
 // Per matrix entry (row r, column l) of one level, the facts ext+i looks up:
 // strong (IF_S), func[l] == func[r] (IF_SAME), l a C point (IF_C), l == r
-// (IF_DIAG).  One warp per row, coalesced.
+// (IF_DIAG), a_rr < 0 or NaN (IF_NEG: abar keeps the positive a_rl, else the
+// negative ones).  L lanes per row, coalesced.
 template <int L>
 __global__ void k_entry_flags(int n, const int32_t* __restrict__ rp,
-                              const int32_t* __restrict__ ci, const uint8_t* __restrict__ S,
+                              const int32_t* __restrict__ ci, const double* __restrict__ v,
+                              const uint8_t* __restrict__ S,
                               const int32_t* __restrict__ cf, const int32_t* __restrict__ func,
                               uint8_t* __restrict__ ef) {
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int r = (int)(g / L), lane = (int)(g % L);
-  if (r >= n) return;
-  const int fr = func[r];
-  for (int t = rp[r] + lane; t < rp[r + 1]; t += L) {
+  const bool valid = r < n;
+  const unsigned base = (threadIdx.x & 31) & ~(unsigned)(L - 1);
+  const unsigned smask = L == 32 ? 0xffffffffu : (((1u << L) - 1u) << base);
+  const int t0 = valid ? rp[r] : 0, t1 = valid ? rp[r + 1] : 0, fr = valid ? func[r] : 0;
+  bool neg = false;
+  for (int t = t0 + lane; t < t1; t += L)
+    if (ci[t] == r) neg = !d_ge0(v[t]);
+  const int sign = (__ballot_sync(0xffffffffu, neg) & smask) ? IF_NEG : 0;
+  for (int t = t0 + lane; t < t1; t += L) {
     const int l = ci[t];
     ef[t] = (uint8_t)((S[t] ? IF_S : 0) | (func[l] == fr ? IF_SAME : 0) |
-                      (cf[l] == 1 ? IF_C : 0) | (l == r ? IF_DIAG : 0));
+                      (cf[l] == 1 ? IF_C : 0) | (l == r ? IF_DIAG : 0) | sign);
   }
 }
 
@@ -1199,7 +1207,7 @@ template <int L>
 __global__ void k_interp_sizes(int n, const int32_t* __restrict__ rp,
                                const int32_t* __restrict__ ci, const uint8_t* __restrict__ ef,
                                const int32_t* __restrict__ cf, int32_t* __restrict__ ub,
-                               int* stage) {
+                               int32_t* __restrict__ kcnt, int* stage) {
   const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int i = (int)(g / L), lane = (int)(g % L);
   const bool valid = i < n;
@@ -1209,7 +1217,7 @@ __global__ void k_interp_sizes(int n, const int32_t* __restrict__ rp,
     const int len = rp[i + 1] - rp[i];
     if (len > ld_volatile_i32(stage + 2)) atomicMax(stage + 2, len);
   }
-  int u = 0, sz = 0;
+  int u = 0, sz = 0, nk = 0;
   if (valid && cf[i] != 1) {
     const int t1 = rp[i + 1];
     for (int t0 = rp[i]; t0 < t1; t0 += L) {
@@ -1221,7 +1229,9 @@ __global__ void k_interp_sizes(int n, const int32_t* __restrict__ rp,
         else { j = ci[t]; sf = true; }
       }
       // the row's lanes scan each strong F neighbour's row together
-      for (unsigned m = __ballot_sync(smask, sf); m; m &= m - 1) {
+      const unsigned sfm = __ballot_sync(smask, sf);
+      nk += __popc(sfm);
+      for (unsigned m = sfm; m; m &= m - 1) {
         const int k = __shfl_sync(smask, j, __ffs(m) - 1);
         const int b = rp[k], e = rp[k + 1];
         if (lane == 0) sz += e - b;
@@ -1236,6 +1246,7 @@ __global__ void k_interp_sizes(int n, const int32_t* __restrict__ rp,
   }
   if (valid && lane == 0) {
     ub[i] = u;
+    kcnt[i] = nk;
     if (sz > ld_volatile_i32(stage)) atomicMax(stage, sz);
     if (u > ld_volatile_i32(stage + 1)) atomicMax(stage + 1, u);  // largest candidate count
   }
@@ -2139,6 +2150,7 @@ __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int 
 
 inline int nblk(long long n) { return n > 0 ? ceil_div(n, kT) : 1; }
 
+#include "interp_group.cuh"
 #include "spgemm_acc.cuh"
 
 // Stream-ordered scratch of one setup step, given back when the step ends.
@@ -2192,6 +2204,40 @@ cptr_status acc_run(cptr_ctx* c, AccArgs a, int cls, int from, int rows, bool sh
                         c->stream>>>(a, from));
       return CPTR_OK;
     }
+  }
+}
+
+template <int G, int H, int Q, int TC, int KC>
+cptr_status ix_launch(cptr_ctx* c, IxArgs a, int cls, int from, int rows) {
+  constexpr int W = 2, R = W * 32 / G;
+  auto kern = k_interp_group<G, H, Q, TC, KC, W>;
+  const size_t smem = sizeof(IxRow<H, Q, TC, KC>) * R;
+  if (smem > 48 * 1024) CTX_CUDA(c, raise_smem_limit(c, (const void*)kern));
+  KL(c, kern<<<std::min(ceil_div(rows, R), 1 << 20), 32 * W, smem, c->stream>>>(a, cls, from));
+  return CPTR_OK;
+}
+// Every class's rows, ncls[k] of them (host copy of a.ncls, read before); on
+// return ncls[kIxClasses] counts the rows left for k_interp_row (pcnt = -1).
+cptr_status ix_run_all(cptr_ctx* c, IxArgs a, int* ncls) {
+  int done[kIxClasses] = {};
+  for (;;) {  // a class launched after a smaller one also takes the rows it deferred
+    bool left = false;
+    for (int k = 0; k < kIxClasses; ++k) {
+      if (ncls[k] <= done[k]) continue;
+      left = true;
+      const int rows = ncls[k] - done[k];
+      cptr_status st = k == 0 ? ix_launch<16, 64, 40, 96, 16>(c, a, k, done[k], rows)
+                     : k == 1 ? ix_launch<32, 128, 64, 256, 40>(c, a, k, done[k], rows)
+                              : ix_launch<32, 512, 256, 1536, 128>(c, a, k, done[k], rows);
+      if (st) return st;
+      done[k] = -1;  // launched: done up to the count read below
+    }
+    if (!left) return CPTR_OK;
+    CTX_CUDA(c, cudaMemcpyAsync(ncls, a.ncls, (kIxClasses + 1) * sizeof(int),
+                                cudaMemcpyDeviceToHost, c->stream));
+    CTX_CUDA(c, cudaStreamSynchronize(c->stream));
+    for (int k = 0; k < kIxClasses; ++k)
+      if (done[k] < 0) done[k] = ncls[k];
   }
 }
 
@@ -2845,10 +2891,26 @@ cptr_status setup_amg(cptr_ctx* c) {
         CTX_CUDA(c, cudaMemsetAsync(flags, 0, 5 * sizeof(int), c->stream));
         uint8_t* ef;
         CTX_ALLOC(c, ef, uint8_t, nnz + 1, true);
-        ROW_LAUNCH(c, row_lanes(n, L->A.nnz), n, k_entry_flags, n, L->A.rp, L->A.ci, S, L->cf,
-                   L->func, ef);
+        ROW_LAUNCH(c, row_lanes(n, L->A.nnz), n, k_entry_flags, n, L->A.rp, L->A.ci, L->A.v, S,
+                   L->cf, L->func, ef);
+        Scratch scr(c);
+        int32_t* kcnt = scr.get<int32_t>(n + 1);
+        if (!kcnt) return CPTR_ERR_NOMEM;
         ROW_LAUNCH(c, row_lanes(n, L->A.nnz), n, k_interp_sizes, n, L->A.rp, L->A.ci, ef, L->cf,
-                   ub, flags + 2);
+                   ub, kcnt, flags + 2);
+        // by lane groups; hooks 3, 4, 5: every F point starts in class 0, 1, 2
+        const bool grouped = !c->force_fallback && (c->interp_path == 0 || c->interp_path > 2);
+        IxArgs ix{n, pmax, L->A.rp, L->A.ci, L->A.v, ef, cidx, pcnt, pcol, pval, nullptr, nullptr};
+        int ncls[kIxClasses + 1] = {};
+        if (grouped) {
+          ix.rows = scr.get<int32_t>((size_t)(kIxClasses + 1) * n);
+          ix.ncls = scr.get<int>(kIxClasses + 1);
+          if (!ix.rows || !ix.ncls) return CPTR_ERR_NOMEM;
+          CTX_CUDA(c, cudaMemsetAsync(ix.ncls, 0, sizeof(ncls), c->stream));
+          KL(c, k_ix_bin<<<nblk(n), kT, 0, c->stream>>>(ix, L->cf, ub, kcnt, c->interp_path - 3));
+          CTX_CUDA(c, cudaMemcpyAsync(ncls, ix.ncls, sizeof(ncls), cudaMemcpyDeviceToHost,
+                                      c->stream));
+        }
         // largest staging size, candidate count and row length, in one read
         int mx3[3] = {0, 0, 0};
         CTX_CUDA(c, cudaMemcpyAsync(mx3, flags + 2, 3 * sizeof(int), cudaMemcpyDeviceToHost,
@@ -2871,31 +2933,32 @@ cptr_status setup_amg(cptr_ctx* c) {
         // hold a few dozen columns, and a row whose set exceeds the table is
         // deferred like any row that does not fit)
         const int hs_s = std::min(hsz, 512), rl_s = std::min(rl, 512), kc_s = std::min(kcap, 512);
-        // short rows (every phase fits one warp's lanes a few times): one warp
-        // per row with a small ordered-sum table, so that more rows are resident
-        const bool narrow = c->interp_path == 0 && rl_s <= 32 && kc_s <= 128;
         const int tmin = 256;  // the table holds |Chat|+1 terms per strong F neighbour
-        const int ithr = narrow ? 32 : (hs_s >= 2048 ? 256 : 128);
         size_t smem = interp_layout(hs_s, rl_s, kc_s, tmin).total;
-        int over = (smem > kMaxSmem || c->force_fallback) ? 1 : 0;
+        int over = ((!grouped && smem > kMaxSmem) || c->force_fallback) ? 1 : 0;
         if (!over) {
-          CTX_CUDA(c, cudaFuncSetAttribute(k_interp_row<false>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)kMaxSmem));
           int* dfl;
           CTX_ALLOC(c, dfl, int, 3, true);
           CTX_CUDA(c, cudaMemsetAsync(dfl, 0, 3 * sizeof(int), c->stream));
-          if (c->interp_path == 2) {  // every row to the global-scratch pass
-            CTX_CUDA(c, cudaMemsetAsync(pcnt, 0xff, sizeof(int32_t) * n, c->stream));
-            CTX_CUDA(c, cudaMemcpyAsync(dfl, &n, sizeof(int), cudaMemcpyHostToDevice, c->stream));
-          } else
-            KL(c, k_interp_row<false><<<n, ithr, smem, c->stream>>>(
-                    n, hs_s, ub, rl_s, kc_s, tmin, L->A.rp, L->A.ci, L->A.v, ef, L->cf, L->func, cidx,
-                    pmax, pcnt, pcol, pval, dfl, nullptr, nullptr, nullptr));
           int ndef = 0;
-          CTX_CUDA(c, cudaMemcpyAsync(&ndef, dfl, sizeof(int), cudaMemcpyDeviceToHost,
-                                      c->stream));
-          CTX_CUDA(c, cudaStreamSynchronize(c->stream));
+          if (grouped) {
+            st = ix_run_all(c, ix, ncls);
+            if (st) return st;
+            ndef = ncls[kIxClasses];
+          } else if (c->interp_path == 2) {  // every row to the global-scratch pass
+            CTX_CUDA(c, cudaMemsetAsync(pcnt, 0xff, sizeof(int32_t) * n, c->stream));
+            ndef = n;
+          } else {
+            CTX_CUDA(c, cudaFuncSetAttribute(k_interp_row<false>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kMaxSmem));
+            KL(c, k_interp_row<false><<<n, hs_s >= 2048 ? 256 : 128, smem, c->stream>>>(
+                      n, hs_s, ub, rl_s, kc_s, tmin, L->A.rp, L->A.ci, L->A.v, ef, L->cf, L->func,
+                      cidx, pmax, pcnt, pcol, pval, dfl, nullptr, nullptr, nullptr));
+            CTX_CUDA(c, cudaMemcpyAsync(&ndef, dfl, sizeof(int), cudaMemcpyDeviceToHost,
+                                        c->stream));
+            CTX_CUDA(c, cudaStreamSynchronize(c->stream));
+          }
           if (ndef > 0) {
             int32_t *drows, *dbytes;
             long long* goff;

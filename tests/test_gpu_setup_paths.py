@@ -53,3 +53,18 @@ def test_spgemm_classes(P, monkeypatch, name, path, pmax):
     assert len(got) == len(ref)
     for a, b in zip(got, ref):
         np.testing.assert_array_equal(a, b)
+
+
+# path 3, 4, 5: every F point starts in the first, second and third class of the
+# lane-group kernels (rows that do not fit move up), 1: wide blocks
+@pytest.mark.parametrize("pmax", [1, 4, 12])
+@pytest.mark.parametrize("path", ["1", "3", "4", "5"])
+@pytest.mark.parametrize("name", list(SYSTEMS))
+def test_interp_classes(P, monkeypatch, name, path, pmax):
+    s = SYSTEMS[name]()
+    ref = hierarchy(P, s, pmax=pmax)
+    monkeypatch.setenv("CPTR_INTERP_PATH", path)
+    got = hierarchy(P, s, pmax=pmax)
+    assert len(got) == len(ref)
+    for a, b in zip(got, ref):
+        np.testing.assert_array_equal(a, b)

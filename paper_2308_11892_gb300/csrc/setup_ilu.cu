@@ -114,45 +114,43 @@ __device__ bool inv4(const double* M, double* out) {
   return true;
 }
 
-// The same Gauss-Jordan inversion executed by a full warp: lane 8*r + k holds
-// entry k of row r of the augmented 4x8 matrix [M | I].  Pivot choice, row
-// swap, scaling and elimination perform exactly the operations of inv4 on the
-// same values, so the result is identical.  M and out may alias (shared memory).
-__device__ bool inv4_warp(const double* M, double* out) {
-  const int lane = threadIdx.x & 31, r = lane >> 3, k = lane & 7;
-  double a = (k < 4) ? M[r * 4 + k] : (k - 4 == r ? 1.0 : 0.0);
-  bool ok = true;
-  for (int c = 0; c < 4; ++c) {
-    // candidate pivots a[rr][c], rr = c..3 (first maximum wins, as in inv4);
-    // |x| and the comparisons run on bit patterns with IEEE results (a NaN
-    // never wins; a NaN first candidate is kept)
-    int p = c;
-    unsigned long long best = dmag(__shfl_sync(0xffffffffu, a, 8 * c + c));
-    for (int rr = c + 1; rr < 4; ++rr) {
-      const unsigned long long v = dmag(__shfl_sync(0xffffffffu, a, 8 * rr + c));
+// The same inversion of two blocks by one warp, in place: lane 4 r + c of each
+// half holds entry (r, c) and returns that of the inverse.  Pivots as in inv4;
+// the columns, exchanged instead of an augmented half, are put back at the end.
+// ok is false for the half whose block has no finite nonzero pivot.
+__device__ __forceinline__ double inv4_pair(double a, bool* ok) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int hl = threadIdx.x & 15, r = hl >> 2, c = hl & 3;
+  int piv[4];
+  *ok = true;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    // candidate pivots a[rr][k], rr >= k (first maximum wins; |x| and the
+    // comparisons run on bit patterns with IEEE results: a NaN never wins, a NaN
+    // first candidate is kept)
+    int p = k;
+    unsigned long long best = dmag(__shfl_sync(FULL, a, 4 * k + k, 16));
+#pragma unroll
+    for (int rr = k + 1; rr < 4; ++rr) {
+      const unsigned long long v = dmag(__shfl_sync(FULL, a, 4 * rr + k, 16));
       if (v > best && v <= 0x7ff0000000000000ull && best <= 0x7ff0000000000000ull) {
         best = v;
         p = rr;
       }
     }
-    if (best == 0 || best >= 0x7ff0000000000000ull) ok = false;  // !(best > 0) || !isfinite
-    // swap rows c and p
-    double from_p = __shfl_sync(0xffffffffu, a, 8 * p + k);
-    double from_c = __shfl_sync(0xffffffffu, a, 8 * c + k);
-    if (r == c) a = from_p;
-    else if (r == p) a = from_c;
-    // scale row c by its pivot
-    double d = __shfl_sync(0xffffffffu, a, 8 * c + c);
-    if (r == c) a = a / d;
-    // eliminate column c from the other rows
-    double pivrow = __shfl_sync(0xffffffffu, a, 8 * c + k);
-    double f = __shfl_sync(0xffffffffu, a, 8 * r + c);
-    if (r != c) a = a - f * pivrow;
+    if (best == 0 || best >= 0x7ff0000000000000ull) *ok = false;
+    piv[k] = p;
+    a = __shfl_sync(FULL, a, 4 * (r == k ? p : r == p ? k : r) + c, 16);  // rows k and p
+    const double d = __shfl_sync(FULL, a, 4 * k + k, 16);
+    const double t = (c == k ? 1.0 : a) / d;
+    const double row = __shfl_sync(FULL, t, 4 * k + c, 16);
+    const double f = __shfl_sync(FULL, a, 4 * r + k, 16);
+    a = r == k ? t : (c == k ? 0.0 : a) - f * row;
   }
-  __syncwarp();
-  if (k >= 4) out[r * 4 + (k - 4)] = a;
-  __syncwarp();
-  return __all_sync(0xffffffffu, ok);
+#pragma unroll
+  for (int k = 3; k >= 0; --k)
+    a = __shfl_sync(FULL, a, 4 * r + (c == k ? piv[k] : c == piv[k] ? k : c), 16);
+  return a;
 }
 
 __device__ __forceinline__ bool wait_flag(const int* flag, int epoch, int* status) {
@@ -231,113 +229,223 @@ __global__ void __launch_bounds__(256) k_ilu_factor(int npos, const int32_t* __r
   }
 }
 
-// Same factorisation with the row staged in shared memory: one warp per row,
-// row i's blocks and columns loaded once (while its dependencies finish), and
-// for every dependency k one parallel load of inv(U_kk) and of row k's upper
-// part.  Column matches are found lane-parallel by binary search; the block
-// products keep the sequential order of the definition (same results).  Rows
-// longer than kRowMax blocks set *overflow and are left to k_ilu_factor.
+// The same factorisation, two rows per warp: sixteen lanes per row, lane 4 r + c
+// holding entry (r, c) of a 4x4 block, both rows (neighbours in the schedule, so
+// of one level) in lockstep; products are fused, except in the inversion, whose
+// pivots decide what is singular.  The kernel is bound by FP64 issue on wide
+// levels, where an instruction costs the same for 16 lanes as for 32, and by the
+// chain flag - inv(U_kk) - L_ik - update - ... - inversion - flag on narrow ones,
+// where a row's first dependency may be its last to come: the rows share every
+// FP64 instruction; the row's blocks and the columns that row i and its
+// dependencies share (pattern only) are ready before the first wait; the flags
+// are read together, and a published dependency's blocks are loaded while the one
+// before it is worked on; one release publishes the row.  Rows longer than maxrow
+// blocks do not come here.  200x200x100 grid 34.8 -> 9.8 ms, 1M-point cloud 21.7 ->
+// 17.5 ms, 64x64x32 grid 2.2 -> 1.5 ms (one row per warp, a dependency's loads after
+// its own flag; two rows per warp without the look-ahead: 25.9 ms on the cloud).
 constexpr int kRowMax = 32;
 constexpr int kFacWarps = 4;
-struct FacWarpSmem {
-  double bi[kRowMax][16];
-  double bk[kRowMax][16];
-  double uinv[16];
-  int ci[kRowMax];
-  int ck[kRowMax];
-  int match[kRowMax];
-  int mt[kRowMax];
+constexpr int kAhead = 2;  // shared blocks of a dependency loaded ahead
+struct FacRow {  // shared memory of one row: byte offsets, cap shared columns listed
+  int cj, ms, mp, mt, cap, bytes;
 };
+inline FacRow fac_row(int maxrow) {
+  FacRow L;
+  L.cap = 4 * maxrow;
+  L.cj = 128 * maxrow;
+  L.ms = L.cj + 4 * maxrow;
+  L.mp = L.ms + 4 * (maxrow + 1);
+  L.mt = L.mp + 4 * L.cap;
+  L.bytes = (L.mt + L.cap + 15) & ~15;
+  return L;
+}
 
-__global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_staged(
-    int npos, const int32_t* __restrict__ ord, const int32_t* __restrict__ rp,
+__global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_pair(
+    int npos, FacRow Ly, const int32_t* __restrict__ ord, const int32_t* __restrict__ rp,
     const int32_t* __restrict__ ci, const int32_t* __restrict__ diag, double* LU, int* done,
-    int epoch, Ctl* ctl, int* overflow) {
+    int epoch, Ctl* ctl) {
   extern __shared__ __align__(16) unsigned char fsm[];
-  FacWarpSmem& W = reinterpret_cast<FacWarpSmem*>(fsm)[threadIdx.x >> 5];
-  int lane = threadIdx.x & 31;
-  int r = (lane >> 2) & 3, c = lane & 3;
-  bool act = lane < 16;
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31, half = lane >> 4, hl = lane & 15, r = hl >> 2, c = hl & 3;
+  unsigned char* base = fsm + (size_t)(threadIdx.x >> 4) * Ly.bytes;
+  double* bi = reinterpret_cast<double*>(base);
+  int* cj = reinterpret_cast<int*>(base + Ly.cj);
+  int* ms = reinterpret_cast<int*>(base + Ly.ms);  // first shared column of each dependency
+  int* mp = reinterpret_cast<int*>(base + Ly.mp);  // its block of row k
+  unsigned char* mt = base + Ly.mt;                // its block of row i
+  const unsigned ngroups = (unsigned)((npos + 1) >> 1);
+  int* const status = &ctl->status;
   for (;;) {
-    unsigned item = 0;
-    if (lane == 0) item = atomicAdd(&ctl->fac_ctr, 1u);
-    item = __shfl_sync(0xffffffffu, item, 0);
-    if (item >= (unsigned)npos) return;
-    int i = ord[item];
-    if (i < 0) continue;
-    int t0 = rp[i], t1 = rp[i + 1], ni = t1 - t0, di = diag[i] - t0;
-    if (ni > kRowMax) {
-      if (lane == 0) atomicExch(overflow, 1);
-      continue;  // left for the fallback kernel
-    }
-    if (lane < ni) W.ci[lane] = ci[t0 + lane];
-    for (int q = lane; q < 16 * ni; q += 32) W.bi[q >> 4][q & 15] = LU[16 * (size_t)t0 + q];
+    unsigned g = 0;
+    if (lane == 0) g = atomicAdd(&ctl->fac_ctr, 1u);
+    g = __shfl_sync(FULL, g, 0);
+    if (g >= ngroups) return;
+    const int pos = (int)(2 * g) + half;
+    const int i = pos < npos ? ord[pos] : -1;
+    const int t0 = i >= 0 ? rp[i] : 0, ni = i >= 0 ? rp[i + 1] - t0 : 0;
+    const int di = i >= 0 ? diag[i] - t0 : 0;
+    for (int e = hl; e < ni; e += 16) cj[e] = ci[t0 + e];
+#pragma unroll 4
+    for (int e = 0; e < ni; ++e) bi[16 * e + hl] = LU[16 * (size_t)(t0 + e) + hl];
     __syncwarp();
-    for (int e = 0; e < di; ++e) {
-      int k = W.ci[e];
-      if (lane == 0) wait_flag(done + k, epoch, &ctl->status);
-      __syncwarp();
-      int kd = diag[k], nu = rp[k + 1] - kd - 1;
-      if (nu > kRowMax) nu = kRowMax;  // rows that long are flagged by their own warp
-      if (lane < 16) W.uinv[lane] = __ldcg(LU + 16 * (size_t)kd + lane);
-      if (lane < nu) W.ck[lane] = __ldcg(ci + kd + 1 + lane);
-      for (int q = lane; q < 16 * nu; q += 32)
-        W.bk[q >> 4][q & 15] = __ldcg(LU + 16 * (size_t)(kd + 1) + q);
-      __syncwarp();
-      // L_ik = A_ik inv(U_kk)
-      double s = 0.0;  // (the sum starts at its first product: 0.0 + x only loses -0.0)
-      if (act) {
-        s = W.bi[e][r * 4] * W.uinv[c];
-        for (int q = 1; q < 4; ++q) s += W.bi[e][r * 4 + q] * W.uinv[q * 4 + c];
-      }
-      __syncwarp();
-      if (act) W.bi[e][r * 4 + c] = s;
-      // matches of row i's later columns in row k's upper part (rows hold at
-      // most 32 blocks: one later column per lane), as a compact list
-      {
-        const int t3 = e + 1 + lane;
-        int pos = -1;
-        if (t3 < ni) {
-          int j = W.ci[t3], lo = 0, hi = nu - 1;
+    const int maxd = __reduce_max_sync(FULL, di);
+    // the later columns of row i in the upper part of row k = cj[e], listed from
+    // slot n on; returns their number
+    auto shared_columns = [&](int e, bool act, int n) {
+      const int k = act ? cj[e] : 0, kd = act ? diag[k] : 0, ke = act ? rp[k + 1] : 0;
+      const int maxl = __reduce_max_sync(FULL, act ? ni - e - 1 : 0);
+      int nm = 0;
+      for (int b = 0; b < maxl; b += 16) {
+        const int t3 = e + 1 + b + hl;
+        int at = -1;
+        if (act && t3 < ni) {
+          const int j = cj[t3];
+          int lo = kd + 1, hi = ke - 1;
           while (lo <= hi) {
-            int mid = (lo + hi) >> 1;
-            int x = W.ck[mid];
-            if (x == j) { pos = mid; break; }
+            const int mid = (lo + hi) >> 1, x = ci[mid];
+            if (x == j) { at = mid; break; }
             if (x < j) lo = mid + 1; else hi = mid - 1;
           }
         }
-        const unsigned mm = __ballot_sync(0xffffffffu, pos >= 0);
-        if (pos >= 0) {
-          const int slot = __popc(mm & ((1u << lane) - 1u));
-          W.mt[slot] = t3;
-          W.match[slot] = pos;
+        const unsigned m = (__ballot_sync(FULL, at >= 0) >> (16 * half)) & 0xffffu;
+        const int slot = n + nm + __popc(m & ((1u << hl) - 1u));
+        if (at >= 0 && slot < Ly.cap) {
+          mt[slot] = (unsigned char)t3;
+          mp[slot] = at;
         }
-        __syncwarp();
-        // A_ij -= L_ik U_kj for the matched j, two blocks at a time (lanes
-        // 16..31 take the odd matches): every block still gets its one update
-        // for this k, with the same products in the same order
-        const int nm = __popc(mm), hw = lane >> 4;
-        for (int a = 0; a < nm; a += 2) {
-          const int q3 = a + hw;
-          if (q3 < nm) {
-            const int tt = W.mt[q3], m = W.match[q3];
-            double p = W.bi[e][r * 4] * W.bk[m][c];
-            for (int q = 1; q < 4; ++q) p += W.bi[e][r * 4 + q] * W.bk[m][q * 4 + c];
-            W.bi[tt][r * 4 + c] = W.bi[tt][r * 4 + c] - p;
+        nm += __popc(m);
+      }
+      return nm;
+    };
+    int listed = 0, late = 0;  // dependencies from `late` on did not fit the list
+    {
+      bool fits = true;
+      for (int e = 0; e < maxd; ++e) {
+        const int nm = shared_columns(e, fits && e < di, listed);
+        if (fits && e < di) {
+          fits = listed + nm <= Ly.cap;
+          if (fits) {
+            if (hl == 0) ms[e] = listed;
+            listed += nm;
+            late = e + 1;
           }
         }
-        __syncwarp();
       }
-    }
-    if (!inv4_warp(W.bi[di], W.bi[di])) {
-      if (lane == 0) dev_fail(&ctl->status, DEV_BREAKDOWN);
-      if (lane < 16) W.bi[di][lane] = 0.0;
+      if (hl == 0) ms[late] = listed;
     }
     __syncwarp();
-    for (int q = lane; q < 16 * ni; q += 32) LU[16 * (size_t)t0 + q] = W.bi[q >> 4][q & 15];
-    __threadfence();
+    // published dependencies by bit; every pending flag is read together
+    unsigned pub = 0;
+    auto read_flags = [&] {
+      for (int b = 0; b < maxd; b += 16) {
+        const int e = b + hl;
+        bool f = false;
+        if (e < di && !(pub >> e & 1u)) f = ld_acquire_i32(done + cj[e]) == epoch;
+        pub |= ((__ballot_sync(FULL, f) >> (16 * half)) & 0xffffu) << b;
+      }
+    };
+    // inv(U_kk) and the first kAhead shared blocks of row k for dependency e
+    struct Blocks {
+      double u[4], w[kAhead][4];
+    };
+    auto load = [&](int e, bool act, Blocks& B) {
+      const int kd = act ? diag[cj[e]] : 0;
+      const int m0 = act && e < late ? ms[e] : 0, nm = act && e < late ? ms[e + 1] - m0 : 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) B.u[q] = act ? __ldcg(LU + 16 * (size_t)kd + 4 * q + c) : 0.0;
+#pragma unroll
+      for (int m = 0; m < kAhead; ++m) {
+        const int b = m < nm ? mp[m0 + m] : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          B.w[m][q] = m < nm ? __ldcg(LU + 16 * (size_t)b + 4 * q + c) : 0.0;
+      }
+    };
+    Blocks cur, nxt;
+    bool have = false;  // cur holds dependency e's blocks
+    for (int e = 0; e < maxd; ++e) {
+      const bool act = e < di;
+      // both rows' dependencies published (bounded; a failed solve runs on)
+      for (unsigned s = 0; __any_sync(FULL, act && !(pub >> e & 1u)); ++s) {
+        read_flags();
+        if (s >= 64) __nanosleep(64);  // back off: fewer polls competing with working warps
+        if ((s & 255u) == 255u) {
+          bool stop = ld_volatile_i32(status) != DEV_OK;
+          if (s > CPTR_SPIN_LIMIT) {
+            dev_fail(status, DEV_TIMEOUT);
+            stop = true;
+          }
+          if (__any_sync(FULL, stop)) break;
+        }
+      }
+      __syncwarp();
+      if (!have) load(e, act, cur);
+      // the next dependency's blocks, if they are published, behind this one's work
+      const bool nhave = e + 1 < di && (pub >> (e + 1) & 1u);
+      load(e + 1, nhave, nxt);
+      int m0 = 0, nm = 0;
+      if (act && e < late) {
+        m0 = ms[e];
+        nm = ms[e + 1] - m0;
+      }
+      const bool unlisted = act && e >= late;
+      if (__any_sync(FULL, unlisted)) {
+        const int n = shared_columns(e, unlisted, 0);
+        if (unlisted) nm = n;
+        __syncwarp();
+        if (unlisted)
+          for (int m = 0; m < kAhead; ++m)
+            for (int q = 0; q < 4; ++q)
+              cur.w[m][q] = m < nm ? __ldcg(LU + 16 * (size_t)mp[m] + 4 * q + c) : 0.0;
+      }
+      const int maxm = __reduce_max_sync(FULL, nm);
+      // L_ik = A_ik inv(U_kk)
+      double l = 0.0;
+      if (act) {
+        const double* A = bi + 16 * e + 4 * r;
+        l = A[0] * cur.u[0];
+#pragma unroll
+        for (int q = 1; q < 4; ++q) l = __fma_rn(A[q], cur.u[q], l);
+      }
+      double lr[4];  // row r of L_ik
+#pragma unroll
+      for (int q = 0; q < 4; ++q) lr[q] = __shfl_sync(FULL, l, 4 * r + q, 16);
+      if (act) bi[16 * e + hl] = l;
+      // A_ij -= L_ik U_kj
+      auto update = [&](int m, const double* w) {
+        const int at = m < nm ? 16 * (int)mt[m0 + m] + hl : 0;
+        double x = m < nm ? bi[at] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x = __fma_rn(-lr[q], w[q], x);
+        if (m < nm) bi[at] = x;
+      };
+#pragma unroll
+      for (int m = 0; m < kAhead; ++m)
+        if (m < maxm) update(m, cur.w[m]);
+      for (int m = kAhead; m < maxm; ++m) {
+        double w[4];
+        const int b = m < nm ? mp[m0 + m] : 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) w[q] = m < nm ? __ldcg(LU + 16 * (size_t)b + 4 * q + c) : 0.0;
+        update(m, w);
+      }
+      cur = nxt;
+      have = nhave;
+      __syncwarp();
+    }
+    bool ok;
+    double dv = inv4_pair(i >= 0 ? bi[16 * di + hl] : (r == c ? 1.0 : 0.0), &ok);
+    if (!ok) {
+      dv = 0.0;
+      if (hl == 0) dev_fail(status, DEV_BREAKDOWN);
+    }
+    if (i >= 0) {
+      bi[16 * di + hl] = dv;
+#pragma unroll 4
+      for (int e = 0; e < ni; ++e) LU[16 * (size_t)(t0 + e) + hl] = bi[16 * e + hl];
+    }
     __syncwarp();
-    if (lane == 0) st_release_i32(done + i, epoch);
+    if (hl == 0 && i >= 0) st_release_i32(done + i, epoch);
     __syncwarp();
   }
 }
@@ -496,17 +604,17 @@ cptr_status setup_ilu_factor(cptr_ctx* c) {
   c->fac_epoch += 1;
   CTX_CUDA(c, cudaMemsetAsync(&c->ctl->fac_ctr, 0, sizeof(unsigned), cs(c)));
   int* mrow;
-  CTX_ALLOC(c, mrow, int, 2, true);
-  CTX_CUDA(c, cudaMemsetAsync(mrow, 0, 2 * sizeof(int), cs(c)));
+  CTX_ALLOC(c, mrow, int, 1, true);
+  CTX_CUDA(c, cudaMemsetAsync(mrow, 0, sizeof(int), cs(c)));
   KL(c, k_max_row<<<nblk(N), kT, 0, cs(c)>>>(N, c->rp, mrow));
   int hm = 0;
   CTX_CUDA(c, cudaMemcpyAsync(&hm, mrow, sizeof(int), cudaMemcpyDeviceToHost, cs(c)));
   CTX_CUDA(c, cudaStreamSynchronize(cs(c)));
   if (hm <= kRowMax && !c->force_fallback) {
-    size_t smem = kFacWarps * sizeof(FacWarpSmem);
-    KL(c, k_ilu_factor_staged<<<c->nsm * 8, 32 * kFacWarps, smem, cs(c)>>>(
-              c->npos_f, c->ord_f, c->rp, c->ci, c->diag, c->LU64, c->fac_done, c->fac_epoch,
-              c->ctl, mrow + 1));
+    const FacRow lay = fac_row(hm);
+    KL(c, k_ilu_factor_pair<<<c->nsm * 8, 32 * kFacWarps, (size_t)lay.bytes * 2 * kFacWarps,
+                              cs(c)>>>(c->npos_f, lay, c->ord_f, c->rp, c->ci, c->diag, c->LU64,
+                                       c->fac_done, c->fac_epoch, c->ctl));
   } else {
     KL(c, k_ilu_factor<<<c->nsm * 4, 256, 0, cs(c)>>>(c->npos_f, c->ord_f, c->rp, c->ci,
                                                           c->diag, c->LU64, c->fac_done,

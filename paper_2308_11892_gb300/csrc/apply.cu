@@ -71,13 +71,50 @@ __global__ void k_restrict(int N, const TIN* __restrict__ vbase, const int* jptr
 }
 
 // ------------------------------------------------------------------ V-cycle
-// LANES consecutive lanes cooperate on one row of a scalar CSR operator.
-template <int LANES, class T>
-__device__ __forceinline__ T row_dot(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                     const T* __restrict__ val, const T* __restrict__ x, int i,
-                                     int sl) {
+// LANES consecutive lanes cooperate on one row of a scalar CSR operator.  What
+// binds these kernels is the gathers of x (a 32-byte sector from L2 for each
+// entry that misses L1) and, for short rows, the loads in flight per lane: up to
+// eight lanes, each takes four consecutive entries at a time with 16-byte loads of
+// the columns and values (the finest level of the 200x200x100 grid, 4 lanes: sweep
+// and residual 0.296 -> 0.260 ms); wider, one entry per lane keeps a row's
+// gathers together (level 1 of that grid, 16 lanes: 0.40 against 0.41 ms; with two
+// gathers per entry 0.46 against 0.52).  The
+// 16-byte loads start at multiples of four entries, so that a row's first and last
+// may hold entries of its neighbours (or of the padding every array ends with),
+// which are skipped.  Returns the row's sum in every lane; ok is false for lanes
+// past the last row.
+__device__ __forceinline__ void ld_vals4(const float* p, float* o) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
+}
+__device__ __forceinline__ void ld_vals4(const double* p, double* o) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+  const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+}
+template <int LANES, class T, class X>
+__device__ __forceinline__ T row_sum(bool ok, int i, int sl, const int32_t* __restrict__ rp,
+                                     const int32_t* __restrict__ ci, const T* __restrict__ val,
+                                     X xval) {
   T s = 0;
-  for (int t = rp[i] + sl; t < rp[i + 1]; t += LANES) s += val[t] * x[ci[t]];
+  if (ok) {
+    const int t0 = rp[i], t1 = rp[i + 1];
+    if (LANES > 8) {
+      for (int t = t0 + sl; t < t1; t += LANES) s += val[t] * xval(ci[t]);
+    } else {
+      for (int t = (t0 & ~3) + 4 * sl; t < t1; t += 4 * LANES) {
+        const int4 c4 = __ldg(reinterpret_cast<const int4*>(ci + t));
+        const int j[4] = {c4.x, c4.y, c4.z, c4.w};
+        T a[4], x[4];
+        ld_vals4(val + t, a);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = (t + u >= t0 && t + u < t1) ? xval(j[u]) : T(0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (t + u >= t0 && t + u < t1) s += a[u] * x[u];
+      }
+    }
+  }
 #pragma unroll
   for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
   return s;
@@ -92,15 +129,8 @@ __global__ void k_vc_pre(int n, const int32_t* __restrict__ rp, const int32_t* _
   if (!*active || n <= 0) return;
   long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int i = (int)(g / LANES), sl = (int)(g % LANES);
-  bool ok = i < n;
-  int ii = ok ? i : n - 1;
-  T s = 0;
-  for (int t = rp[ii] + sl; ok && t < rp[ii + 1]; t += LANES) {
-    int j = ci[t];
-    s += val[t] * (dinv[j] * b[j]);
-  }
-#pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
+  const bool ok = i < n;
+  const T s = row_sum<LANES>(ok, i, sl, rp, ci, val, [&](int j) { return dinv[j] * b[j]; });
   if (ok && sl == 0) {
     T bi = b[i];
     x[i] = dinv[i] * bi;
@@ -108,21 +138,21 @@ __global__ void k_vc_pre(int n, const int32_t* __restrict__ rp, const int32_t* _
   }
 }
 
-// y = M x for a scalar CSR M (restriction by R).
+// y = M x for a scalar CSR M (restriction by R), and the next level's first
+// smoothing iterate from zero, y0 = Dinv y, where dinv is given.
 template <int LANES, class T>
 __global__ void k_csr_mv(int n, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                          const T* __restrict__ val, const T* __restrict__ x, T* __restrict__ y,
-                         const int* active) {
+                         const T* __restrict__ dinv, T* __restrict__ y0, const int* active) {
   if (!*active || n <= 0) return;
   long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int i = (int)(g / LANES), sl = (int)(g % LANES);
-  bool ok = i < n;
-  int ii = ok ? i : n - 1;
-  T s = 0;
-  for (int t = rp[ii] + sl; ok && t < rp[ii + 1]; t += LANES) s += val[t] * x[ci[t]];
-#pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
-  if (ok && sl == 0) y[i] = s;
+  const bool ok = i < n;
+  const T s = row_sum<LANES>(ok, i, sl, rp, ci, val, [&](int j) { return x[j]; });
+  if (ok && sl == 0) {
+    y[i] = s;
+    if (dinv) y0[i] = dinv[i] * s;
+  }
 }
 
 // x += P xc (prolongation, at most pmax entries per row).
@@ -147,12 +177,8 @@ __global__ void k_vc_post(int n, const int32_t* __restrict__ rp, const int32_t* 
   if (!*active || n <= 0) return;
   long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int i = (int)(g / LANES), sl = (int)(g % LANES);
-  bool ok = i < n;
-  int ii = ok ? i : n - 1;
-  T s = 0;
-  for (int t = rp[ii] + sl; ok && t < rp[ii + 1]; t += LANES) s += val[t] * xin[ci[t]];
-#pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
+  const bool ok = i < n;
+  const T s = row_sum<LANES>(ok, i, sl, rp, ci, val, [&](int j) { return xin[j]; });
   if (ok && sl == 0) xout[i] = xin[i] + dinv[i] * (b[i] - s);
 }
 
@@ -164,12 +190,8 @@ __global__ void k_vc_resid(int n, const int32_t* __restrict__ rp, const int32_t*
   if (!*active || n <= 0) return;
   long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   int i = (int)(g / LANES), sl = (int)(g % LANES);
-  bool ok = i < n;
-  int ii = ok ? i : n - 1;
-  T s = 0;
-  for (int t = rp[ii] + sl; ok && t < rp[ii + 1]; t += LANES) s += val[t] * x[ci[t]];
-#pragma unroll
-  for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
+  const bool ok = i < n;
+  const T s = row_sum<LANES>(ok, i, sl, rp, ci, val, [&](int j) { return x[j]; });
   if (ok && sl == 0) r[i] = b[i] - s;
 }
 
@@ -544,16 +566,16 @@ void launch_rowkernel_post(int lanes, int n, const Level& L, const T* b, const T
 }
 
 template <class T>
-void launch_csr_mv(int lanes, const DCSR& M, const T* val, const T* x, T* y, const int* active,
-                   cptr_ctx* c) {
+void launch_csr_mv(int lanes, const DCSR& M, const T* val, const T* x, T* y, const T* dinv, T* y0,
+                   const int* active, cptr_ctx* c) {
   cudaStream_t s = c->stream;
   long long thr = (long long)M.n * lanes;
   switch (lanes) {
-    case 2: KL(c, k_csr_mv<2, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, active)); break;
-    case 4: KL(c, k_csr_mv<4, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, active)); break;
-    case 8: KL(c, k_csr_mv<8, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, active)); break;
-    case 16: KL(c, k_csr_mv<16, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, active)); break;
-    default: KL(c, k_csr_mv<32, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, active)); break;
+    case 2: KL(c, k_csr_mv<2, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, dinv, y0, active)); break;
+    case 4: KL(c, k_csr_mv<4, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, dinv, y0, active)); break;
+    case 8: KL(c, k_csr_mv<8, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, dinv, y0, active)); break;
+    case 16: KL(c, k_csr_mv<16, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, dinv, y0, active)); break;
+    default: KL(c, k_csr_mv<32, T><<<nblk(thr), kT, 0, s>>>(M.n, M.rp, M.ci, val, x, y, dinv, y0, active)); break;
   }
 }
 
@@ -605,9 +627,12 @@ void launch_vcycle(cptr_ctx* c, const T* b0, const int* active) {
   for (int l = 0; l < last; ++l) {
     Level& L = c->lev[l];
     const T* b = (l == 0) ? b0 : (const T*)L.b;
-    if (fused_pre) {
+    if (fused_pre && l == 0) {
       // one l1-Jacobi sweep from zero (x = D^-1 b) fused with the residual
       launch_rowkernel_pre<T>(L.lanes, L.A.n, L, b, (T*)L.x, (T*)L.r, active, c);
+    } else if (fused_pre) {
+      // x = D^-1 b came with b from the level above: one gather per entry, not two
+      launch_resid<T>(L.lanes, L.A.n, L, b, (const T*)L.x, (T*)L.r, active, c);
     } else {
       // nu1 sweeps from x = 0 (zero start in r), alternating between t and x
       // so that the last one writes x, then r = b - A x
@@ -627,7 +652,10 @@ void launch_vcycle(cptr_ctx* c, const T* b0, const int* active) {
     }
     double ravg = L.R.n ? (double)L.R.nnz / L.R.n : 1.0;
     int rl = ravg <= 8 ? 2 : ravg <= 20 ? 4 : ravg <= 48 ? 8 : 16;
-    launch_csr_mv<T>(rl, L.R, (const T*)L.Rv, (const T*)L.r, (T*)c->lev[l + 1].b, active, c);
+    Level& Ln = c->lev[l + 1];
+    const bool first = fused_pre && l + 1 < last;  // (the coarsest level has no smoother)
+    launch_csr_mv<T>(rl, L.R, (const T*)L.Rv, (const T*)L.r, (T*)Ln.b,
+                     first ? (const T*)Ln.dinv : nullptr, (T*)Ln.x, active, c);
   }
   {
     Level& Lc = c->lev[last];

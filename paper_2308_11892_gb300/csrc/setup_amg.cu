@@ -2024,22 +2024,6 @@ __device__ __forceinline__ unsigned gj_rank() {
   return r;
 }
 template <class V>
-__device__ __forceinline__ V gj_remote(const V* local_ptr, unsigned rank) {
-  unsigned la = (unsigned)__cvta_generic_to_shared(local_ptr), ra;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
-  V v;
-  if (sizeof(V) == 8) {
-    unsigned long long x;
-    asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(x) : "r"(ra) : "memory");
-    memcpy(&v, &x, 8);
-  } else {
-    unsigned x;
-    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(x) : "r"(ra) : "memory");
-    memcpy(&v, &x, 4);
-  }
-  return v;
-}
-template <class V>
 __device__ __forceinline__ void gj_push(V* local_ptr, unsigned rank, V v) {
   unsigned la = (unsigned)__cvta_generic_to_shared(local_ptr), ra;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(rank));
@@ -2053,14 +2037,23 @@ __device__ __forceinline__ void gj_push(V* local_ptr, unsigned rank, V v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(ra), "r"(x) : "memory");
   }
 }
-// Gauss-Jordan with partial pivoting of [M | I] on one cluster, each CTA
-// holding a slice of w columns in shared memory.  At step k the CTA owning
-// column k picks the pivot with one warp (largest |a_rk|, ties to the smaller
-// row), and pushes the pivot row index, the pivot and the column-k factors of
-// the swapped matrix into every CTA's double-buffered arrays; one cluster
-// barrier publishes them (passing step k-1's barrier means every CTA has
-// finished step k-2, so buffer k & 1 is free).  Each CTA then swaps, scales
-// and eliminates its own slice.
+// Gauss-Jordan inversion with partial pivoting on one cluster, in place: each CTA
+// holds a slice of w columns in shared memory, a finished column is replaced by
+// the column of the inverse that elimination grows beside it, and the columns are
+// put back in order at the end (the row exchanges, undone as column exchanges).
+// At step k the CTA owning column k picks the pivot with one warp (largest
+// |a_rk|, ties to the smaller row), and pushes the pivot row index, the pivot and
+// the column-k factors of the swapped matrix into every CTA's double-buffered
+// arrays; one cluster barrier publishes them (passing step k-1's barrier means
+// every CTA has finished step k-2, so buffer k & 1 is free).  Each CTA then swaps,
+// scales and eliminates its own slice.
+//
+// The steps are a serial chain; each is bound by its CTA's FP64 rate (n w updates
+// at two per cycle) beside the barrier's latency, so an update is one fused
+// multiply-add, zeros are tested on the integer pipes, every column of every
+// slice is active, and no index is divided.  n = 208:
+// 1.40 -> 0.80 ms, n = 146: 0.68 -> 0.44 ms ([M | I] beside each other, an
+// FP64 compare, multiply and subtraction per element, before).
 __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int w,
                                                                      const double* __restrict__ M,
                                                                      double* __restrict__ inv,
@@ -2068,51 +2061,56 @@ __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int 
   extern __shared__ __align__(16) double gjs[];
   double* S = gjs;                      // n x w slice
   double* fcolb = gjs + (size_t)n * w;  // 2 x n pushed column-k factors
+  int* piv_row = reinterpret_cast<int*>(fcolb + 2 * (size_t)n);  // n pivot rows
+  int* place = piv_row + n;             // n: column of the inverse held by a column
   __shared__ int s_p[2];
   __shared__ double s_piv[2];
   __shared__ int own_p;
   const unsigned q = gj_rank();
-  const int tid = threadIdx.x;
-  const int c0 = (int)q * w, W = 2 * n;
-  const int wq = max(0, min(w, W - c0));
-  for (size_t x = tid; x < (size_t)n * w; x += blockDim.x) {
-    int r = (int)(x / w), cc = (int)(x % w);
-    S[x] = cc < wq ? M[(size_t)r * W + c0 + cc] : 0.0;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = (int)q * w, wq = max(0, min(w, n - c0));
+  // element x = r w + c of the slice, walked by steps of the block size
+  const int dr = kGjThreads / w, dc = kGjThreads % w, r0 = tid / w, cc0 = tid % w;
+  for (int r = r0, cc = cc0; r < n;) {
+    S[r * w + cc] = cc < wq ? M[(size_t)r * 2 * n + c0 + cc] : 0.0;
+    r += dr;
+    cc += dc;
+    if (cc >= w) { cc -= w; ++r; }
   }
   __syncthreads();
-  gj_cluster_sync();  // every slice filled before any push or DSMEM access
+  gj_cluster_sync();  // every slice filled before any push
   bool failed = false;
   for (int k = 0; k < n; ++k) {
     const unsigned o = (unsigned)(k / w);  // owner of column k
-    const int b = k & 1;
+    const int b = k & 1, kc = k - c0;
     if (q == o) {
-      const int kc = k - c0;
       if (tid < 32) {
-        double best = -1.0;
+        unsigned long long best = 0;  // |a| by its bits (a NaN never wins)
         int bi = n;
         for (int r = k + tid; r < n; r += 32) {
-          const double a = fabs(S[(size_t)r * w + kc]);
-          if (a > best) { best = a; bi = r; }
+          const unsigned long long a = dmag(S[r * w + kc]);
+          if (a <= 0x7ff0000000000000ull && (bi == n || a > best)) { best = a; bi = r; }
         }
         for (int off = 16; off > 0; off >>= 1) {
-          const double ov = __shfl_xor_sync(0xffffffffu, best, off);
+          const unsigned long long ov = __shfl_xor_sync(0xffffffffu, best, off);
           const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-          if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+          if (oi < n && (bi == n || ov > best || (ov == best && oi < bi))) { best = ov; bi = oi; }
         }
-        if (tid == 0) own_p = (best > 0.0 && isfinite(best) && bi < n) ? bi : -1;
+        if (tid == 0) own_p = (best > 0 && best < 0x7ff0000000000000ull && bi < n) ? bi : -1;
       }
       __syncthreads();
       const int p = own_p;
-      // column k of the matrix with rows k and p swapped, with 0 at row k
-      for (int x = tid; x < kGjCtas * n; x += blockDim.x) {
-        const int dst = x / n, r = x % n;
+      // column k of the matrix with rows k and p swapped, with 0 at row k; warp d
+      // pushes it to CTA d
+      static_assert(kGjThreads / 32 == kGjCtas, "one warp per CTA of the cluster");
+      for (int r = lane; r < n; r += 32) {
         const int src = (r == k) ? p : (r == p ? k : r);
-        const double f = (r == k || p < 0) ? 0.0 : S[(size_t)src * w + kc];
-        gj_push(&fcolb[(size_t)b * n + r], (unsigned)dst, f);
+        const double f = (r == k || p < 0) ? 0.0 : S[src * w + kc];
+        gj_push(&fcolb[(size_t)b * n + r], (unsigned)warp, f);
       }
-      if (tid < kGjCtas) {
-        gj_push(&s_p[b], (unsigned)tid, p);
-        gj_push(&s_piv[b], (unsigned)tid, p >= 0 ? S[(size_t)p * w + kc] : 0.0);
+      if (lane == 0) {
+        gj_push(&s_p[b], (unsigned)warp, p);
+        gj_push(&s_piv[b], (unsigned)warp, p >= 0 ? S[p * w + kc] : 0.0);
       }
     }
     gj_cluster_sync();
@@ -2120,31 +2118,46 @@ __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int 
     if (p < 0) { failed = true; break; }  // every CTA reads the same value
     const double piv = s_piv[b];
     const double* fcol = fcolb + (size_t)b * n;
-    // swap rows k and p, scale row k (the pivot row), from column k on
-    const int cstart = max(0, k - c0);
-    for (int cc = cstart + tid; cc < wq; cc += blockDim.x) {
-      double vk = S[(size_t)k * w + cc], vp = S[(size_t)p * w + cc];
-      if (p != k) S[(size_t)p * w + cc] = vk;
-      S[(size_t)k * w + cc] = vp / piv;
+    if (tid == 0) piv_row[k] = p;
+    // swap rows k and p, scale row k; column k starts its column of the inverse
+    for (int cc = tid; cc < wq; cc += kGjThreads) {
+      const double vk = S[k * w + cc], vp = S[p * w + cc];
+      if (p != k) S[p * w + cc] = vk;
+      S[k * w + cc] = (cc == kc ? 1.0 : vp) / piv;
     }
     __syncthreads();
-    const int nc = wq - cstart;
-    if (nc > 0) {
-      for (size_t x = tid; x < (size_t)n * nc; x += blockDim.x) {
-        const int r = (int)(x / nc), cc = cstart + (int)(x % nc);
-        const double f = fcol[r];
-        if (f != 0.0) S[(size_t)r * w + cc] -= f * S[(size_t)k * w + cc];
+    for (int r = r0, cc = cc0; r < n;) {
+      const double f = fcol[r];
+      if (!d_eq0(f)) {
+        const double a = cc == kc ? 0.0 : S[r * w + cc];
+        S[r * w + cc] = __fma_rn(-f, S[k * w + cc], a);
       }
+      r += dr;
+      cc += dc;
+      if (cc >= w) { cc -= w; ++r; }
     }
     __syncthreads();
   }
   if (failed && q == 0 && tid == 0) dev_fail(status, DEV_BREAKDOWN);
   gj_cluster_sync();  // no CTA leaves while another may still write into it
   if (failed) return;
-  for (size_t x = tid; x < (size_t)n * wq; x += blockDim.x) {
-    const int r = (int)(x / wq), cc = (int)(x % wq);
-    const int col = c0 + cc;
-    if (col >= n) inv[(size_t)r * n + (col - n)] = S[(size_t)r * w + cc];
+  // column j of the inverse is column idx[j] here: the exchanges undone, last first
+  if (tid == 0) {
+    int* idx = reinterpret_cast<int*>(fcolb);  // (the factors are done with)
+    for (int j = 0; j < n; ++j) idx[j] = j;
+    for (int k = n - 1; k >= 0; --k) {
+      const int t = idx[k];
+      idx[k] = idx[piv_row[k]];
+      idx[piv_row[k]] = t;
+    }
+    for (int j = 0; j < n; ++j) place[idx[j]] = j;
+  }
+  __syncthreads();
+  for (int r = r0, cc = cc0; r < n;) {
+    if (cc < wq) inv[(size_t)r * n + place[c0 + cc]] = S[r * w + cc];
+    r += dr;
+    cc += dc;
+    if (cc >= w) { cc -= w; ++r; }
   }
 }
 
@@ -3088,8 +3101,9 @@ cptr_status setup_amg(cptr_ctx* c) {
       // one cluster holding the whole augmented matrix when it fits, else one block
       bool clustered = false;
       {
-        const int w = (2 * nn + kGjCtas - 1) / kGjCtas;
-        const size_t csmem = sizeof(double) * ((size_t)nn * w + 2 * (size_t)nn);
+        const int w = (nn + kGjCtas - 1) / kGjCtas;
+        const size_t csmem = sizeof(double) * ((size_t)nn * w + 2 * (size_t)nn) +
+                             2 * sizeof(int) * (size_t)nn;
         if (csmem <= 200 * 1024) {
           CTX_CUDA(c, cudaFuncSetAttribute(k_gauss_jordan_cluster,
                                            cudaFuncAttributeNonPortableClusterSizeAllowed, 1));

@@ -182,8 +182,8 @@ cptr_status cptr_setup(cptr_ctx* c);
 cptr_status cptr_solve(cptr_ctx* c, const double* rhs, double* x, double tol, int maxit,
                        cptr_info* info);
 
-/* Solves n small systems in one launch: one thread block per system runs the
- * whole flexible GMRES(restart) loop with the Eq. 3 preconditioner on the
+/* Solves n small systems at once on the device: one thread block, or a cluster of
+ * up to eight, per system runs the whole flexible GMRES(restart) loop with the Eq. 3 preconditioner on the
  * device (block SpMV, restriction, V-cycle, correction, ILU(0) level by level,
  * CGS2, Givens rotations, restarts, true residual), with no host
  * synchronisation per iteration; the systems advance concurrently.  The same
@@ -199,7 +199,7 @@ cptr_status cptr_solve(cptr_ctx* c, const double* rhs, double* x, double tol, in
  * Runs on the stream of ctxs[0] after every context's earlier work; returns
  * CPTR_OK when all converged, else the first failure (a breakdown before
  * CPTR_ERR_MAXIT); every x[k] is written.  Meant for systems of up to tens of
- * thousands of cells: one block per system. */
+ * thousands of cells: one block or cluster per system. */
 cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const double* const* rhs,
                              double* const* x, double tol, int maxit, cptr_info* infos);
 

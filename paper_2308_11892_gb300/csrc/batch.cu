@@ -2,12 +2,13 @@
 //
 // A small system (thousands of cells) leaves most of the GPU idle in the
 // per-system path, whose Krylov loop launches a few dozen kernels per
-// iteration and reads a host flag at every restart.  Here one thread block
-// runs the whole flexible GMRES(m) loop of one system on the device, with the
+// iteration and reads a host flag at every restart.  Here one thread block, or a
+// cluster of up to eight, runs the whole flexible GMRES(m) loop of one system on
+// the device, with the
 // Eq. 3 preconditioner (Quasi-IMPES restriction, the system-AMG V-cycle, the
 // correction, the ILU(0) solves level by level, the combination), the outer
 // block SpMV, CGS2 with Givens rotations, the back substitution, restarts and
-// the true residual, separated by block barriers only; a grid of such blocks
+// the true residual, separated by block or cluster barriers only; a grid of them
 // advances every system of the batch at once.  Each system reads its own
 // context's hierarchy, factors and work vectors (built by cptr_setup), and
 // every sum has a fixed order that does not depend on the batch: a system's
@@ -17,6 +18,7 @@
 #include <string>
 #include <cmath>
 #include <cstdio>
+#include <cstdlib>
 #include <vector>
 
 #include "common.cuh"
@@ -24,7 +26,7 @@
 
 namespace {
 
-constexpr int kBT = 512;        // threads per system
+constexpr int kBT = 512;        // threads per block
 constexpr int kBMaxLev = 25;    // AMG levels
 constexpr int kBMaxM = 32;      // restart length
 
@@ -34,6 +36,7 @@ struct BLevel {
   const void* Av;    // apply precision
   const void* dinv;  // apply precision
   int nc;            // rows of the next level (R: nc x n, P: n x nc)
+  int lanes, rlanes; // lanes per row of A and of R (by their mean row lengths)
   const int32_t *Rrp, *Rci;
   const void* Rv;
   const int32_t *Prp, *Pci;
@@ -56,207 +59,562 @@ struct alignas(16) BSys {
   const void *Uv, *Dinv;
   double *V, *w, *x, *b;
   void* Z;
+  unsigned spin;  // reads a dependency wait makes before it gives up
+  int* fail;      // set when one did
   BLevel lev[kBMaxLev];
 };
 
 struct BOut {
-  int iters, status;
+  int iters, status, fail;
   double rel_resid;
 };
 
-// Sum of v over the block in a fixed order (warps, then warp sums in order);
-// every thread returns the total.
-__device__ double bsum(double v, double* red) {
-  v = warp_sum(v);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();  // red is free (a previous call may still be reading it)
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  for (int q = 0; q < (int)(blockDim.x >> 5); ++q) t += red[q];
-  return t;
+// A system runs on one cluster of 1, 2, 4 or 8 blocks (see cptr_solve_batch):
+// every loop over rows is dealt over the cluster's threads, and a phase ends at a
+// cluster barrier, which also makes the blocks' writes to global memory visible.
+// A row's sum never depends on the dealing, and the dots and norms are cut into
+// kParts slices of the rows whatever the number of blocks, so the result is the
+// same on any cluster size.
+//
+// One block is bound by its SM's FP64 rate (outer SpMV, CGS2) and by memory
+// latency (V-cycle rows, ILU(0) levels); the cluster divides the first by its
+// size, and the levels read what does not depend on the level before ahead of
+// the barrier.
+struct Team {
+  int rank, size;  // block of the cluster, blocks in it
+  int tid, threads;
+  __device__ __forceinline__ Team() {
+    unsigned r, n;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+    rank = (int)r;
+    size = (int)n;
+    tid = rank * kBT + (int)threadIdx.x;
+    threads = size * kBT;
+  }
+  __device__ __forceinline__ void sync() const {
+    if (size == 1) {
+      __syncthreads();
+    } else {
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                   "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+  }
+};
+// A double of another block's shared memory.
+__device__ __forceinline__ double team_read(const double* own, int rank) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(own), r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  double v;
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
 }
 
-// The row loops below load four entries before summing their products (in
-// entry order, the same sums as an entry-by-entry loop).  One SM carries a
-// whole system here, so the FP64 parts (the outer SpMV, CGS2, norms) run at
-// that SM's FP64 rate, which bounds them; the FP32 preconditioner waits on
-// block barriers and memory latency.
+constexpr int kParts = 32;
+// Partial sums of a reduction, this block's slices; two of them alternate, so that
+// a block may start the next reduction while another still reads this one.
+struct Partials {
+  double v[2][kParts * (kBMaxM + 1)];
+  int flip;
+};
+
+// out[l] = V_l . w for l < nc (V_l = V + l n), the same in every block: a warp sums
+// G columns over one slice, the slices are combined by a shuffle tree.
+template <int G>
+__device__ __forceinline__ void part_dot(const double* V, size_t n, const double* w, int lo,
+                                         int hi, double* out) {
+  const int lane = threadIdx.x & 31;
+  double acc[G];
+#pragma unroll
+  for (int u = 0; u < G; ++u) acc[u] = 0.0;
+#pragma unroll 4
+  for (int i = lo + lane; i < hi; i += 32) {
+    const double wi = w[i];
+#pragma unroll
+    for (int u = 0; u < G; ++u) acc[u] += V[(size_t)u * n + i] * wi;
+  }
+#pragma unroll
+  for (int u = 0; u < G; ++u) {
+    const double s = warp_sum(acc[u]);
+    if (lane == 0) out[u] = s;
+  }
+}
+__device__ __noinline__ void team_dots(const Team& t, Partials& P, const double* V, const double* w, int n,
+                          int nc, double* out) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kBT / 32;
+  const int mine = kParts / t.size;
+  const int per = ((n + kParts - 1) / kParts + 31) & ~31;
+  const int groups = (nc + 3) / 4;
+  double* part = P.v[P.flip];
+  for (int unit = warp; unit < mine * groups; unit += nw) {
+    const int p = unit / groups, g = unit % groups;
+    const int lo = min(n, (t.rank * mine + p) * per), hi = min(n, lo + per);
+    double* o = part + p * (kBMaxM + 1) + 4 * g;
+    const double* Vg = V + (size_t)(4 * g) * n;
+    switch (min(4, nc - 4 * g)) {
+      case 1: part_dot<1>(Vg, n, w, lo, hi, o); break;
+      case 2: part_dot<2>(Vg, n, w, lo, hi, o); break;
+      case 3: part_dot<3>(Vg, n, w, lo, hi, o); break;
+      default: part_dot<4>(Vg, n, w, lo, hi, o); break;
+    }
+  }
+  t.sync();
+  for (int l = warp; l < nc; l += nw) {
+    const double s = warp_sum(team_read(part + (lane % mine) * (kBMaxM + 1) + l, lane / mine));
+    if (lane == 0) out[l] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) P.flip ^= 1;
+  __syncthreads();
+}
+
+// w -= V h over the first nc columns, four elements per thread at a time (their
+// loads overlap; each element takes its columns in order).
+__device__ __noinline__ void team_update(const Team& t, const double* V, double* w, int n, int nc,
+                                         const double* h) {
+  for (int i0 = t.tid; i0 < n; i0 += 4 * t.threads) {
+    double wi[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) wi[u] = i0 + u * t.threads < n ? w[i0 + u * t.threads] : 0.0;
+    const double* v = V + i0;
+#pragma unroll 2
+    for (int l = 0; l < nc; ++l, v += n) {
+      const double hl = h[l];
+      double x[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = i0 + u * t.threads < n ? v[u * t.threads] : 0.0;
+#pragma unroll
+      for (int u = 0; u < 4; ++u) wi[u] -= hl * x[u];
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (i0 + u * t.threads < n) w[i0 + u * t.threads] = wi[u];
+  }
+}
+
+// The row loops below load several entries before summing their products (in
+// entry order, the same sums as an entry-by-entry loop).
+
+__device__ __forceinline__ void ld4x(const double* p, double* o) {
+  const double2 a = *reinterpret_cast<const double2*>(p);
+  const double2 b = *(reinterpret_cast<const double2*>(p) + 1);
+  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+}
+__device__ __forceinline__ void ld4x(const float* p, float* o) {
+  const float4 a = *reinterpret_cast<const float4*>(p);
+  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
+}
+__device__ __forceinline__ void ld4x(const float* p, double* o) {  // (off the FP64 pipe)
+  float f[4];
+  ld4x(p, f);
+  widen<4>(f, o);
+}
 
 // y = A x (4x4 blocks, FP64 accumulation in block order), y = b - A x when b
 template <class TX>
-__device__ void bspmv(const BSys& S, const TX* __restrict__ x, const double* __restrict__ b,
-                      double* __restrict__ y) {
+__device__ __noinline__ void bspmv(const Team& t, const BSys& S, const TX* x, const double* b, double* y) {
   const int n4 = 4 * S.N;
   const int32_t* __restrict__ rp = S.rp;
   const int32_t* __restrict__ ci = S.ci;
   const double* __restrict__ v = S.v;
-  for (int g = threadIdx.x; g < n4; g += blockDim.x) {
+  for (int g = t.tid; g < n4; g += t.threads) {
     const int i = g >> 2, r = g & 3;
     double acc = 0.0;
-    int t = rp[i];
-    const int t1 = rp[i + 1];
-    for (; t + 4 <= t1; t += 4) {
+    int k = rp[i];
+    const int k1 = rp[i + 1];
+    for (; k + 4 <= k1; k += 4) {
       int j[4];
       double a[4][4], xv[4][4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) j[u] = ci[t + u];
+      for (int u = 0; u < 4; ++u) j[u] = ci[k + u];
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          a[u][q] = v[16 * (size_t)(t + u) + 4 * r + q];
-          xv[u][q] = (double)x[4 * (size_t)j[u] + q];
-        }
+      for (int u = 0; u < 4; ++u) {
+        ld4(v + 16 * (size_t)(k + u) + 4 * r, a[u]);
+        ld4x(x + 4 * (size_t)j[u], xv[u]);
+      }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc = fma(a[u][q], xv[u][q], acc);
     }
-    for (; t < t1; ++t) {
-      const double* a = v + 16 * (size_t)t + 4 * r;
-      const TX* xj = x + 4 * (size_t)ci[t];
-      acc = fma(a[0], (double)xj[0], acc);
-      acc = fma(a[1], (double)xj[1], acc);
-      acc = fma(a[2], (double)xj[2], acc);
-      acc = fma(a[3], (double)xj[3], acc);
+    for (; k < k1; ++k) {
+      double a[4], xv[4];
+      ld4(v + 16 * (size_t)k + 4 * r, a);
+      ld4x(x + 4 * (size_t)ci[k], xv);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc = fma(a[q], xv[q], acc);
     }
     y[g] = b ? b[g] - acc : acc;
   }
 }
 
-// sum over row i of a CSR operator of val * x, in entry order
-template <class T>
-__device__ __forceinline__ T row_sum(const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
-                                     const T* __restrict__ val, const T* __restrict__ x, int i) {
-  T s = 0;
-  int t = rp[i];
-  const int t1 = rp[i + 1];
-  for (; t + 4 <= t1; t += 4) {
-    int j[4];
-    T a[4], xv[4];
+// f(i, sum) for every row i < n of a CSR operator, sum = its val * x: L lanes per
+// row (by the operator's mean row length), each summing its entries in order,
+// then a shuffle tree.
+template <int L, class T, class F>
+__device__ __forceinline__ void rows_as(const Team& t, int n, const int32_t* __restrict__ rp,
+                                        const int32_t* __restrict__ ci,
+                                        const T* __restrict__ val, const T* x, F f) {
+  const int sl = threadIdx.x & (L - 1);
+  // whole warps: the lanes of a warp meet at the shuffles
+  const int per = t.threads / L;
+  for (int i0 = 0; i0 < n; i0 += per) {
+    const int i = i0 + t.tid / L;
+    T s = 0;
+    if (i < n) {
+      const int t1 = rp[i + 1];
+      for (int k = rp[i] + sl; k < t1; k += 4 * L) {
+        int j[4];
+        T a[4], xv[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      j[u] = ci[t + u];
-      a[u] = val[t + u];
+        for (int u = 0; u < 4; ++u)
+          if (k + u * L < t1) {
+            j[u] = ci[k + u * L];
+            a[u] = val[k + u * L];
+          }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u * L < t1) xv[u] = x[j[u]];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (k + u * L < t1) s += a[u] * xv[u];
+      }
     }
 #pragma unroll
-    for (int u = 0; u < 4; ++u) xv[u] = x[j[u]];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) s += a[u] * xv[u];
+    for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, L);
+    if (i < n && sl == 0) f(i, s);
   }
-  for (; t < t1; ++t) s += val[t] * x[ci[t]];
-  return s;
+}
+template <class T, class F>
+__device__ __forceinline__ void rows(const Team& t, int n, int lanes,
+                                     const int32_t* __restrict__ rp,
+                                     const int32_t* __restrict__ ci, const T* __restrict__ val,
+                                     const T* x, F f) {
+  // (about four entries per lane: fewer leave too few loads in flight)
+  if (lanes <= 2) rows_as<2>(t, n, rp, ci, val, x, f);
+  else if (lanes <= 4) rows_as<4>(t, n, rp, ci, val, x, f);
+  else rows_as<16>(t, n, rp, ci, val, x, f);
 }
 
 // r = b - A x on one AMG level (scalar CSR, apply precision)
 template <class T>
-__device__ void lresid(const BLevel& L, const T* __restrict__ b, const T* __restrict__ x,
-                       T* __restrict__ r) {
-  const int32_t* __restrict__ rp = L.Arp;
-  const int32_t* __restrict__ ci = L.Aci;
-  const T* __restrict__ av = (const T*)L.Av;
-  const int n = L.n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) r[i] = b[i] - row_sum<T>(rp, ci, av, x, i);
+__device__ __noinline__ void lresid(const Team& t, const BLevel& L, const T* b, const T* x, T* r) {
+  rows<T>(t, L.n, L.lanes, L.Arp, L.Aci, (const T*)L.Av, x, [=](int i, T s) { r[i] = b[i] - s; });
 }
 
 // xout = xin + D_l1^-1 (b - A xin): one l1-Jacobi sweep
 template <class T>
-__device__ void lsweep(const BLevel& L, const T* __restrict__ b, const T* __restrict__ xin,
-                       T* __restrict__ xout) {
-  const int32_t* __restrict__ rp = L.Arp;
-  const int32_t* __restrict__ ci = L.Aci;
-  const T* __restrict__ av = (const T*)L.Av;
-  const T* __restrict__ dv = (const T*)L.dinv;
-  const int n = L.n;
-  for (int i = threadIdx.x; i < n; i += blockDim.x)
-    xout[i] = xin[i] + dv[i] * (b[i] - row_sum<T>(rp, ci, av, xin, i));
+__device__ __noinline__ void lsweep(const Team& t, const BLevel& L, const T* b, const T* xin, T* xout) {
+  const T* dv = (const T*)L.dinv;
+  rows<T>(t, L.n, L.lanes, L.Arp, L.Aci, (const T*)L.Av, xin,
+          [=](int i, T s) { xout[i] = xin[i] + dv[i] * (b[i] - s); });
 }
 
-}  // namespace
-
-namespace {
+// b_{l+1} = R r and x += P xc
+template <class T>
+__device__ __noinline__ void lrestrict(const Team& t, const BLevel& L, const T* r, T* bn) {
+  const int32_t *rp = L.Rrp, *ci = L.Rci;
+  const T* rv = (const T*)L.Rv;
+  auto f = [=](int i, T s) { bn[i] = s; };
+  if (L.rlanes <= 2) rows_as<2>(t, L.nc, rp, ci, rv, r, f);
+  else rows_as<8>(t, L.nc, rp, ci, rv, r, f);
+}
+template <class T>
+__device__ __noinline__ void lprolong(const Team& t, const BLevel& L, const T* xc, T* x) {
+  rows_as<2>(t, L.n, L.Prp, L.Pci, (const T*)L.Pv, xc, [=](int i, T s) { x[i] += s; });
+}
 
 // One V(nu_pre, nu_post) cycle with l1-Jacobi from a zero guess on the
 // system's hierarchy: b0 (level 0 right-hand side) -> zc.
 template <class T>
-__device__ void bvcycle(const BSys& S, const T* b0) {
+__device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) {
   const int last = S.nlev - 1;
   for (int l = 0; l < last; ++l) {
     const BLevel& L = S.lev[l];
     const T* b = l == 0 ? b0 : (const T*)L.b;
     T* x = (T*)L.x;
-    T* t = (T*)L.t;
+    T* tt = (T*)L.t;
     if (S.nu_pre == 0) {
-      for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] = 0;
+      for (int i = t.tid; i < L.n; i += t.threads) x[i] = 0;
     } else {
       // first sweep from zero: x = D^-1 b; the others alternate so the last writes x
-      T* dst = ((S.nu_pre - 1) % 2 == 0) ? x : t;
+      T* dst = ((S.nu_pre - 1) % 2 == 0) ? x : tt;
       const T* dv = (const T*)L.dinv;
-      for (int i = threadIdx.x; i < L.n; i += blockDim.x) dst[i] = dv[i] * b[i];
+      for (int i = t.tid; i < L.n; i += t.threads) dst[i] = dv[i] * b[i];
       const T* src = dst;
       for (int k = 1; k < S.nu_pre; ++k) {
-        __syncthreads();
-        T* d2 = ((S.nu_pre - 1 - k) % 2 == 0) ? x : t;
-        lsweep<T>(L, b, src, d2);
+        t.sync();
+        T* d2 = ((S.nu_pre - 1 - k) % 2 == 0) ? x : tt;
+        lsweep<T>(t, L, b, src, d2);
         src = d2;
       }
     }
-    __syncthreads();
-    lresid<T>(L, b, x, (T*)L.r);
-    __syncthreads();
+    t.sync();
+    lresid<T>(t, L, b, x, (T*)L.r);
+    t.sync();
     // b_{l+1} = R r
-    const T* rv = (const T*)L.Rv;
-    const T* r = (const T*)L.r;
     T* bn = (T*)S.lev[l + 1].b;
-    for (int i = threadIdx.x; i < L.nc; i += blockDim.x) bn[i] = row_sum<T>(L.Rrp, L.Rci, rv, r, i);
-    __syncthreads();
+    lrestrict<T>(t, L, (const T*)L.r, bn);
+    t.sync();
   }
   {
-    // coarsest level: x = Cinv b in FP64
+    // coarsest level: x = Cinv b in FP64, one warp per row, lanes over the columns,
+    // then a fixed shuffle tree
     const BLevel& Lc = S.lev[last];
     const T* b = last == 0 ? b0 : (const T*)Lc.b;
     T* xo = last == 0 ? (T*)S.zc : (T*)Lc.x;
     const int n = Lc.n;
     const double* __restrict__ Cinv = S.Cinv;
     const int lane = threadIdx.x & 31;
-    // one warp per row, lanes over the columns, then a fixed shuffle tree
-    for (int i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5) {
+    for (int i = t.tid >> 5; i < n; i += t.threads >> 5) {
       double s = 0.0;
       for (int q = lane; q < n; q += 32) s += Cinv[(size_t)i * n + q] * (double)b[q];
       s = warp_sum(s);
       if (lane == 0) xo[i] = (T)s;
     }
-    __syncthreads();
+    t.sync();
   }
   for (int l = last - 1; l >= 0; --l) {
     const BLevel& L = S.lev[l];
     const T* b = l == 0 ? b0 : (const T*)L.b;
     const T* xc = (l + 1 == last) ? (const T*)S.lev[l + 1].x : (const T*)S.lev[l + 1].x2;
     T* x = (T*)L.x;
-    T* t = (T*)L.t;
+    T* tt = (T*)L.t;
     T* out = l == 0 ? (T*)S.zc : (T*)L.x2;
-    const T* pv = (const T*)L.Pv;
-    for (int i = threadIdx.x; i < L.n; i += blockDim.x) x[i] += row_sum<T>(L.Prp, L.Pci, pv, xc, i);
-    __syncthreads();
+    lprolong<T>(t, L, xc, x);
+    t.sync();
     if (S.nu_post == 0) {
-      for (int i = threadIdx.x; i < L.n; i += blockDim.x) out[i] = x[i];
+      for (int i = t.tid; i < L.n; i += t.threads) out[i] = x[i];
     } else {
       const T* src = x;
       for (int k = 0; k < S.nu_post; ++k) {
-        T* dst = (k == S.nu_post - 1) ? out : (src == x ? t : x);
-        lsweep<T>(L, b, src, dst);
-        __syncthreads();
+        T* dst = (k == S.nu_post - 1) ? out : (src == x ? tt : x);
+        lsweep<T>(t, L, b, src, dst);
+        if (k + 1 < S.nu_post) t.sync();
         src = dst;
       }
     }
+    t.sync();
+  }
+}
+
+// The ILU(0) solves, one quad per row (lane r: component r), with the library's
+// rounding sequence.  A level is a few dozen rows, so a solve is the latency of its
+// levels, one after the other.
+//
+// One block (tri_solve) separates the levels by its barrier, and everything but the
+// solutions of earlier levels is on its way before a row is worked on: a row's
+// number and block range three levels ahead, its blocks to L2 two ahead and to
+// registers one ahead, behind the level's own gather, which they would delay in
+// front of it.  On a cluster a barrier that publishes global memory costs about
+// 5 us, so there (tri_solve_poll) the rows are dealt over the cluster's quads in
+// schedule order and wait for their dependencies' values instead (a sentinel until
+// they are written, read a bounded number of times); a quad has a row every few
+// levels and reads it ahead while it waits.  The quads take their rows in order and
+// the blocks of a cluster run together, so each wait ends: a 32k-point cloud (405
+// levels) on eight blocks, 7 iterations, 41.5 ms with a barrier per level, 25 ms so.
+struct RowMeta {
+  int p, i, kb, ke;
+};
+__device__ __forceinline__ RowMeta row_meta(int p, int pe, const int32_t* __restrict__ ord,
+                                            const int32_t* __restrict__ rp) {
+  RowMeta m{p, -1, 0, 0};
+  if (p < pe) {
+    m.i = ord[p];
+    m.kb = rp[p];
+    m.ke = rp[p + 1];
+  }
+  return m;
+}
+template <class T>
+struct TriRow {
+  static constexpr int kPre = sizeof(T) == 4 ? 6 : 3;  // dependencies read ahead (registers)
+  int p, i, kb, ke;
+  T acc;
+  int j[kPre];
+  T f[kPre][4];
+};
+template <class T>
+__device__ __forceinline__ void row_data(TriRow<T>& R, const RowMeta& m,
+                                         const int32_t* __restrict__ ci,
+                                         const T* __restrict__ F, const T* rhs, int r) {
+  R.p = m.p;
+  R.i = m.i;
+  R.kb = R.ke = 0;
+  R.acc = 0;
+  if (m.i < 0) return;
+  R.kb = m.kb;
+  R.ke = m.ke;
+  R.acc = rhs[4 * (size_t)m.i + r];
+#pragma unroll
+  for (int u = 0; u < TriRow<T>::kPre; ++u)
+    if (m.kb + u < m.ke) {
+      R.j[u] = ci[m.kb + u];
+      ld4(F + 16 * (size_t)(m.kb + u) + 4 * r, R.f[u]);
+    }
+}
+// the row's right-hand side minus its blocks times the solutions, in block order
+template <class T>
+__device__ __forceinline__ T row_finish(const TriRow<T>& R, const int32_t* __restrict__ ci,
+                                        const T* __restrict__ F, const T* y, int r) {
+  T acc = R.acc;
+  T x[TriRow<T>::kPre][4];
+#pragma unroll
+  for (int u = 0; u < TriRow<T>::kPre; ++u)
+    if (R.kb + u < R.ke) ld4x(y + 4 * (size_t)R.j[u], x[u]);
+#pragma unroll
+  for (int u = 0; u < TriRow<T>::kPre; ++u)
+    if (R.kb + u < R.ke) acc = sub_rn(acc, dot4(R.f[u], x[u]));
+  for (int k = R.kb + TriRow<T>::kPre; k < R.ke; k += 3) {
+    T f[3][4], xx[3][4];
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (k + u < R.ke) {
+        ld4(F + 16 * (size_t)(k + u) + 4 * r, f[u]);
+        ld4x(y + 4 * (size_t)ci[k + u], xx[u]);
+      }
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+      if (k + u < R.ke) acc = sub_rn(acc, dot4(f[u], xx[u]));
+  }
+  return acc;
+}
+// Forward: y = L^-1 rhs.  Backward (UPPER): y = U^-1 rhs and z = P zc + y.
+template <class T, bool UPPER>
+__device__ __noinline__ void tri_solve(const Team& t, const BSys& S, const T* rhs, T* y, T* z) {
+  const int32_t* __restrict__ off = UPPER ? S.offb : S.offf;
+  const int32_t* __restrict__ ord = UPPER ? S.ordb : S.ordf;
+  const int32_t* __restrict__ rp = UPPER ? S.Urp : S.Lrp;
+  const int32_t* __restrict__ ci = UPPER ? S.Uci : S.Lci;
+  const T* __restrict__ F = (const T*)(UPPER ? S.Uv : S.Lv);
+  const int nl = UPPER ? S.nlb : S.nlf;
+  const int r = threadIdx.x & 3, quad = t.tid >> 2, nquad = t.threads >> 2;
+  const unsigned qmask = 0xFu << ((threadIdx.x & 31) & ~3);
+  const int q0 = (threadIdx.x & 31) & ~3;
+  // level lv: positions [o0, o1), the next ones [o1, o2), [o2, o3), [o3, o4)
+  int o0 = off[0], o1 = off[1], o2 = off[min(2, nl)], o3 = off[min(3, nl)];
+  TriRow<T> R;
+  row_data<T>(R, row_meta(o0 + quad, o1, ord, rp), ci, F, rhs, r);
+  RowMeta m1 = row_meta(o1 + quad, o2, ord, rp), m2 = row_meta(o2 + quad, o3, ord, rp);
+  for (int lv = 0; lv < nl; ++lv) {
+    for (int p = o0 + quad;;) {
+      T d[4] = {0, 0, 0, 0}, y1 = 0;
+      if (UPPER && R.i >= 0) {
+        // inv(U_ii) and the first-stage part, beside the gather
+        ld4((const T*)S.Dinv + 16 * (size_t)R.p + 4 * r, d);
+        if (S.first) {
+          const T* zc = (const T*)S.zc;
+          if (r == S.e0) y1 = zc[S.ne * (size_t)R.i];
+          else if (S.ne == 2 && r == S.e1) y1 = zc[2 * (size_t)R.i + 1];
+        }
+      }
+      T acc = R.i >= 0 ? row_finish(R, ci, F, y, r) : T(0);
+      if (UPPER) {
+        T s4[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s4[q] = __shfl_sync(qmask, acc, q0 + q);
+        acc = dot4(d, s4);
+      }
+      if (R.i >= 0) {
+        y[4 * (size_t)R.i + r] = acc;
+        if (UPPER) z[4 * (size_t)R.i + r] = y1 + acc;
+      }
+      p += nquad;
+      if (p >= o1) break;
+      row_data<T>(R, row_meta(p, o1, ord, rp), ci, F, rhs, r);
+    }
+    // in flight behind the barrier: the next level's row, the row numbers three
+    // levels ahead, and the blocks two levels ahead on their way to L2
+    row_data<T>(R, m1, ci, F, rhs, r);
+    const int o4 = off[min(lv + 4, nl)];
+    for (int k = m2.kb + r; k < m2.ke; k += 4) {
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(F + 16 * (size_t)k));
+      if (sizeof(T) == 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(F + 16 * (size_t)k + 8));
+    }
+    if (UPPER && m2.i >= 0 && r == 0)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"((const T*)S.Dinv + 16 * (size_t)m2.p));
+    m1 = m2;
+    m2 = row_meta(o3 + quad, o4, ord, rp);
+    o0 = o1; o1 = o2; o2 = o3; o3 = o4;
     __syncthreads();
   }
 }
 
+// The same solves on a cluster; forward: y_next becomes the sentinel.
+template <class T, bool UPPER>
+__device__ __noinline__ void tri_solve_poll(const Team& t, const BSys& S, const T* rhs, T* y,
+                                            T* y_next, T* z) {
+  const int32_t* __restrict__ ord = UPPER ? S.ordb : S.ordf;
+  const int32_t* __restrict__ rp = UPPER ? S.Urp : S.Lrp;
+  const int32_t* __restrict__ ci = UPPER ? S.Uci : S.Lci;
+  const T* __restrict__ F = (const T*)(UPPER ? S.Uv : S.Lv);
+  constexpr int K = sizeof(T) == 4 ? 4 : 3;  // dependencies read together
+  const int npos = UPPER ? S.offb[S.nlb] : S.offf[S.nlf];
+  const int r = threadIdx.x & 3, quad = t.tid >> 2, nquad = t.threads >> 2;
+  const unsigned qmask = 0xFu << ((threadIdx.x & 31) & ~3);
+  const int q0 = (threadIdx.x & 31) & ~3;
+  for (int p = quad; p < npos; p += nquad) {
+    const int i = ord[p];
+    if (i < 0) continue;
+    const int kb = rp[p], ke = rp[p + 1];
+    T acc = rhs[4 * (size_t)i + r], y1 = 0, d[4];
+    if (UPPER) {
+      // inv(U_ii) and the first-stage part
+      ld4((const T*)S.Dinv + 16 * (size_t)p + 4 * r, d);
+      if (S.first) {
+        const T* zc = (const T*)S.zc;
+        if (r == S.e0) y1 = zc[S.ne * (size_t)i];
+        else if (S.ne == 2 && r == S.e1) y1 = zc[2 * (size_t)i + 1];
+      }
+    }
+    for (int k = kb; k < ke; k += K) {
+      const T* yp[K];
+      T f[K][4], x[K][4];
+      unsigned todo = 0;
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (k + u < ke) {
+          yp[u] = y + 4 * (size_t)ci[k + u];
+          ld4(F + 16 * (size_t)(k + u) + 4 * r, f[u]);
+          todo |= 1u << u;
+        }
+      for (unsigned s = 0; todo; ++s) {
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+          if (todo >> u & 1u) ld_volatile4(yp[u], x[u]);
+#pragma unroll
+        for (int u = 0; u < K; ++u)
+          if ((todo >> u & 1u) && !is_sentinel(x[u][0]) && !is_sentinel(x[u][1]) &&
+              !is_sentinel(x[u][2]) && !is_sentinel(x[u][3]))
+            todo &= ~(1u << u);
+        if (!todo) break;
+        if (s + 1 >= S.spin) {
+          atomicExch(S.fail, 1);
+          break;
+        }
+        if ((s & 255u) == 255u && ld_volatile_i32(S.fail)) break;
+      }
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (k + u < ke) acc = sub_rn(acc, dot4(f[u], x[u]));
+    }
+    if (UPPER) {
+      T s4[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) s4[q] = __shfl_sync(qmask, acc, q0 + q);
+      acc = dot4(d, s4);
+    }
+    st_volatile(y + 4 * (size_t)i + r, desentinel(acc));
+    if (UPPER) z[4 * (size_t)i + r] = y1 + acc;
+    else y_next[4 * (size_t)i + r] = sentinel_of(T(0));
+  }
+  t.sync();
+}
+
 // z = M^-1 v (Eq. 3) for the FP64 vector v; z in the apply precision.
 template <class T>
-__device__ void bprecond(const BSys& S, const double* v, T* z) {
+__device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double* v, T* z) {
   const int N = S.N;
   T* rhat = (T*)S.rhat;
   T* zc = (T*)S.zc;
@@ -266,7 +624,7 @@ __device__ void bprecond(const BSys& S, const double* v, T* z) {
   if (S.first) {
     // Quasi-IMPES restriction: rhat_i = v_i[e] - W_i v_i[h]
     const T* W = (const T*)S.Wt;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+    for (int i = t.tid; i < N; i += t.threads) {
       const double* rv = v + 4 * (size_t)i;
       const T* w = W + 4 * (size_t)i;
       if (S.ne == 2) {
@@ -277,201 +635,132 @@ __device__ void bprecond(const BSys& S, const double* v, T* z) {
         rhat[i] = (T)rv[S.e0] - w[0] * (T)rv[S.h0] - w[1] * (T)rv[S.h1] - w[2] * (T)rv[S.h2];
       }
     }
-    __syncthreads();
-    bvcycle<T>(S, rhat);
+    t.sync();
+    bvcycle<T>(t, S, rhat);
     // correction: r2 = v - A P zc (elliptic columns of A only)
     const T* __restrict__ ae = (const T*)S.AE;
     const int32_t* __restrict__ rp = S.rp;
     const int32_t* __restrict__ ci = S.ci;
     const int ne = S.ne;
-    for (int g = threadIdx.x; g < 4 * N; g += blockDim.x) {
+    for (int g = t.tid; g < 4 * N; g += t.threads) {
       const int i = g >> 2, r = g & 3;
       T acc = 0;
-      int t = rp[i];
-      const int t1 = rp[i + 1];
-      for (; t + 4 <= t1; t += 4) {
+      int k = rp[i];
+      const int k1 = rp[i + 1];
+      for (; k < k1; k += 4) {
         int j[4];
         T a0[4], a1[4], z0[4], z1[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          j[u] = ci[t + u];
-          a0[u] = ae[8 * (size_t)(t + u) + 2 * r];
-          a1[u] = ae[8 * (size_t)(t + u) + 2 * r + 1];
-        }
+        for (int q = 0; q < 4; ++q)
+          if (k + q < k1) {
+            j[q] = ci[k + q];
+            a0[q] = ae[8 * (size_t)(k + q) + 2 * r];
+            a1[q] = ae[8 * (size_t)(k + q) + 2 * r + 1];
+          }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          z0[u] = ne == 2 ? zc[2 * (size_t)j[u]] : zc[j[u]];
-          z1[u] = ne == 2 ? zc[2 * (size_t)j[u] + 1] : T(0);
-        }
+        for (int q = 0; q < 4; ++q)
+          if (k + q < k1) {
+            z0[q] = ne == 2 ? zc[2 * (size_t)j[q]] : zc[j[q]];
+            z1[q] = ne == 2 ? zc[2 * (size_t)j[q] + 1] : T(0);
+          }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (ne == 2) acc += a0[u] * z0[u] + a1[u] * z1[u];
-          else acc += a0[u] * z0[u];
-        }
-      }
-      for (; t < t1; ++t) {
-        const int jj = ci[t];
-        const T* a = ae + 8 * (size_t)t + 2 * r;
-        if (ne == 2) acc += a[0] * zc[2 * (size_t)jj] + a[1] * zc[2 * (size_t)jj + 1];
-        else acc += a[0] * zc[jj];
+        for (int q = 0; q < 4; ++q)
+          if (k + q < k1) {
+            if (ne == 2) acc += a0[q] * z0[q] + a1[q] * z1[q];
+            else acc += a0[q] * z0[q];
+          }
       }
       r2[g] = (T)v[g] - acc;
     }
   } else {
-    for (int g = threadIdx.x; g < 4 * N; g += blockDim.x) r2[g] = (T)v[g];
+    for (int g = t.tid; g < 4 * N; g += t.threads) r2[g] = (T)v[g];
   }
-  __syncthreads();
-  // ILU(0): forward, one level after the other (the library's rounding sequence)
-  const int r = threadIdx.x & 3, quad = threadIdx.x >> 2, nquad = blockDim.x >> 2;
-  const T* Lv = (const T*)S.Lv;
-  for (int lv = 0; lv < S.nlf; ++lv) {
-    for (int p = S.offf[lv] + quad; p < S.offf[lv + 1]; p += nquad) {
-      const int i = S.ordf[p];
-      if (i < 0) continue;
-      T acc = r2[4 * (size_t)i + r];
-      for (int k = S.Lrp[p]; k < S.Lrp[p + 1]; ++k) {
-        T l[4], uj[4];
-        const T* lp = Lv + 16 * (size_t)k + 4 * r;
-        const T* up = u + 4 * (size_t)S.Lci[k];
-        l[0] = lp[0]; l[1] = lp[1]; l[2] = lp[2]; l[3] = lp[3];
-        uj[0] = up[0]; uj[1] = up[1]; uj[2] = up[2]; uj[3] = up[3];
-        acc = sub_rn(acc, dot4(l, uj));
-      }
-      u[4 * (size_t)i + r] = acc;
-    }
-    __syncthreads();
-  }
-  // backward with inv(U_ii), then z = P zc + y2
-  const T* Uv = (const T*)S.Uv;
-  const T* Dv = (const T*)S.Dinv;
-  const unsigned qmask = 0xFu << ((threadIdx.x & 31) & ~3);
-  const int q0 = (threadIdx.x & 31) & ~3;
-  for (int lv = 0; lv < S.nlb; ++lv) {
-    const int pe = S.offb[lv + 1];
-    // uniform rounds: the quads of a warp shuffle together
-    for (int pb = S.offb[lv]; pb < pe; pb += nquad) {
-      const int p = pb + quad;
-      const int i = p < pe ? S.ordb[p] : -1;
-      T acc = 0, d[4] = {0, 0, 0, 0}, y1 = 0;
-      if (i >= 0) {
-        // inv(U_ii) and the first-stage part before the row's sums
-        const T* dp = Dv + 16 * (size_t)p + 4 * r;
-        d[0] = dp[0]; d[1] = dp[1]; d[2] = dp[2]; d[3] = dp[3];
-        if (S.first) {
-          if (r == S.e0) y1 = zc[S.ne * (size_t)i];
-          else if (S.ne == 2 && r == S.e1) y1 = zc[2 * (size_t)i + 1];
-        }
-        acc = u[4 * (size_t)i + r];
-        for (int k = S.Urp[p]; k < S.Urp[p + 1]; ++k) {
-          T a[4], yj[4];
-          const T* ap = Uv + 16 * (size_t)k + 4 * r;
-          const T* yp = y2 + 4 * (size_t)S.Uci[k];
-          a[0] = ap[0]; a[1] = ap[1]; a[2] = ap[2]; a[3] = ap[3];
-          yj[0] = yp[0]; yj[1] = yp[1]; yj[2] = yp[2]; yj[3] = yp[3];
-          acc = sub_rn(acc, dot4(a, yj));
-        }
-      }
-      T s4[4];
-      s4[0] = __shfl_sync(qmask, acc, q0 + 0);
-      s4[1] = __shfl_sync(qmask, acc, q0 + 1);
-      s4[2] = __shfl_sync(qmask, acc, q0 + 2);
-      s4[3] = __shfl_sync(qmask, acc, q0 + 3);
-      if (i >= 0) {
-        const T y = dot4(d, s4);
-        y2[4 * (size_t)i + r] = y;
-        z[4 * (size_t)i + r] = y1 + y;
-      }
-    }
-    __syncthreads();
+  if (t.size > 1)
+    for (int g = t.tid; g < 4 * N; g += t.threads) u[g] = sentinel_of(T(0));
+  t.sync();
+  if (t.size > 1) {
+    tri_solve_poll<T, false>(t, S, r2, u, y2, nullptr);
+    tri_solve_poll<T, true>(t, S, u, y2, nullptr, z);
+  } else {
+    tri_solve<T, false>(t, S, r2, u, nullptr);
+    tri_solve<T, true>(t, S, u, y2, z);
   }
 }
 
-}  // namespace
-
-namespace {
-
-// Flexible GMRES(m) with CGS2 and Givens rotations for system blockIdx.x,
+// Flexible GMRES(m) with CGS2 and Givens rotations for one system per cluster,
 // the same algorithm (and stopping rules) as the per-system driver:
 // convergence when ||b - A x|| <= tol ||b||, iterations = preconditioner
 // applications, a cycle ends at m steps, on convergence of the estimate, at
 // maxit or on an exact breakdown, and the true residual decides whether to
-// start another.
+// start another.  Every block keeps the Hessenberg matrix and takes the same
+// decisions from the same sums.
 template <class T>
 __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict__ sys,
                                                       BOut* __restrict__ out) {
+  const Team t;
+  const int id = blockIdx.x / t.size;
   // the system's descriptor in shared memory: its pointers are then read
   // without a global load, and stores to global memory cannot alias them
   __shared__ BSys S;
   {
-    const int4* src = reinterpret_cast<const int4*>(sys + blockIdx.x);
+    const int4* src = reinterpret_cast<const int4*>(sys + id);
     int4* dst = reinterpret_cast<int4*>(&S);
     for (int k = threadIdx.x; k < (int)(sizeof(BSys) / 16); k += blockDim.x) dst[k] = src[k];
   }
-  __syncthreads();
-  __shared__ double red[kBT / 32];
+  __shared__ Partials P;
+  if (threadIdx.x == 0) P.flip = 0;
+  t.sync();  // (every block of the cluster has started before any reads its memory)
   __shared__ double sH[(kBMaxM + 1) * kBMaxM];  // column j at j*(m+1), rotated
   __shared__ double scs[kBMaxM], ssn[kBMaxM], sg[kBMaxM + 1], sy[kBMaxM], sh1[kBMaxM + 1],
-      sh2[kBMaxM + 1];
+      sh2[kBMaxM + 1], snrm[1];
   __shared__ int s_stop;
   const int n4 = 4 * S.N, m = S.m;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = blockDim.x >> 5;
+  const int tid = threadIdx.x;
   T* Z = (T*)S.Z;
   // ||b||
-  double s = 0.0;
-  for (int i = tid; i < n4; i += blockDim.x) s += S.b[i] * S.b[i];
-  const double bnorm = sqrt(bsum(s, red));
+  team_dots(t, P, S.b, S.b, n4, 1, snrm);
+  const double bnorm = sqrt(snrm[0]);
   const double tol_abs = S.tol * bnorm;
   int iters = 0, status = CPTR_OK;
   double beta = 0.0;
   if (bnorm == 0.0) {
-    for (int i = tid; i < n4; i += blockDim.x) S.x[i] = 0.0;
+    for (int i = t.tid; i < n4; i += t.threads) S.x[i] = 0.0;
   } else {
     for (;;) {
       // r = b - A x into V_0, beta = ||r||
-      bspmv<double>(S, S.x, S.b, S.V);
-      __syncthreads();
-      s = 0.0;
-      for (int i = tid; i < n4; i += blockDim.x) s += S.V[i] * S.V[i];
-      beta = sqrt(bsum(s, red));
+      bspmv<double>(t, S, S.x, S.b, S.V);
+      t.sync();
+      team_dots(t, P, S.V, S.V, n4, 1, snrm);
+      beta = sqrt(snrm[0]);
       if (!isfinite(beta)) { status = CPTR_ERR_BREAKDOWN; break; }
       if (beta <= tol_abs) break;
       if (iters >= S.maxit) { status = CPTR_ERR_MAXIT; break; }
-      for (int i = tid; i < n4; i += blockDim.x) S.V[i] = S.V[i] / beta;
+      for (int i = t.tid; i < n4; i += t.threads) S.V[i] = S.V[i] / beta;
       if (tid == 0) {
         sg[0] = beta;
         for (int l = 1; l <= m; ++l) sg[l] = 0.0;
       }
-      __syncthreads();
+      t.sync();
       int k = 0;
       for (int j = 0; j < m; ++j) {
         const double* vj = S.V + (size_t)j * n4;
         T* zj = Z + (size_t)j * n4;
-        bprecond<T>(S, vj, zj);
-        bspmv<T>(S, zj, nullptr, S.w);
-        __syncthreads();
-        // CGS2: h1 = V^T w; w -= V h1; h2 = V^T w; w -= V h2 (one warp per
-        // column: the FP64 pipe, not the number of warps, bounds these dots)
+        bprecond<T>(t, S, vj, zj);
+        if (t.size > 1 && ld_volatile_i32(S.fail)) {  // (set before the last barrier)
+          status = CPTR_ERR_TIMEOUT;
+          break;
+        }
+        bspmv<T>(t, S, zj, nullptr, S.w);
+        t.sync();
+        // CGS2: h1 = V^T w; w -= V h1; h2 = V^T w; w -= V h2
         for (int pass = 0; pass < 2; ++pass) {
           double* hh = pass == 0 ? sh1 : sh2;
-          const double* __restrict__ wv = S.w;
-          for (int l = warp; l <= j; l += nw) {
-            const double* __restrict__ vl = S.V + (size_t)l * n4;
-            double d = 0.0;
-            for (int i = lane; i < n4; i += 32) d += vl[i] * wv[i];
-            d = warp_sum(d);
-            if (lane == 0) hh[l] = d;
-          }
-          __syncthreads();
-          for (int i = tid; i < n4; i += blockDim.x) {
-            double wi = S.w[i];
-            for (int l = 0; l <= j; ++l) wi -= hh[l] * S.V[(size_t)l * n4 + i];
-            S.w[i] = wi;
-          }
-          __syncthreads();
+          team_dots(t, P, S.V, S.w, n4, j + 1, hh);
+          team_update(t, S.V, S.w, n4, j + 1, hh);
+          t.sync();
         }
-        s = 0.0;
-        for (int i = tid; i < n4; i += blockDim.x) s += S.w[i] * S.w[i];
-        const double hn = sqrt(bsum(s, red));
+        team_dots(t, P, S.w, S.w, n4, 1, snrm);
+        const double hn = sqrt(snrm[0]);
         if (tid == 0) {
           double* col = sH + (size_t)j * (m + 1);
           for (int l = 0; l <= j; ++l) col[l] = sh1[l] + sh2[l];
@@ -503,31 +792,33 @@ __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict_
         if (s_stop) break;
         const double rinv = 1.0 / hn;
         double* vn = S.V + (size_t)(j + 1) * n4;
-        for (int i = tid; i < n4; i += blockDim.x) vn[i] = S.w[i] * rinv;
-        __syncthreads();
+        for (int i = t.tid; i < n4; i += t.threads) vn[i] = S.w[i] * rinv;
+        t.sync();
       }
+      if (status != CPTR_OK) break;
       // y = H^-1 g, x += Z y
       if (tid == 0) {
         for (int i = k - 1; i >= 0; --i) {
-          double t = sg[i];
-          for (int l = i + 1; l < k; ++l) t -= sH[(size_t)l * (m + 1) + i] * sy[l];
-          sy[i] = t / sH[(size_t)i * (m + 1) + i];
+          double s = sg[i];
+          for (int l = i + 1; l < k; ++l) s -= sH[(size_t)l * (m + 1) + i] * sy[l];
+          sy[i] = s / sH[(size_t)i * (m + 1) + i];
         }
       }
       __syncthreads();
-      for (int i = tid; i < n4; i += blockDim.x) {
+      for (int i = t.tid; i < n4; i += t.threads) {
         double xi = S.x[i];
         for (int l = 0; l < k; ++l) xi += sy[l] * (double)Z[(size_t)l * n4 + i];
         S.x[i] = xi;
       }
-      __syncthreads();
+      t.sync();
     }
   }
-  if (tid == 0) {
-    out[blockIdx.x].iters = iters;
-    out[blockIdx.x].status = status;
-    out[blockIdx.x].rel_resid = bnorm > 0.0 ? beta / bnorm : 0.0;
+  if (tid == 0 && t.rank == 0) {
+    out[id].iters = iters;
+    out[id].status = status;
+    out[id].rel_resid = bnorm > 0.0 ? beta / bnorm : 0.0;
   }
+  t.sync();  // no block leaves while another may read its shared memory
 }
 
 }  // namespace
@@ -578,6 +869,8 @@ cptr_status describe(cptr_ctx* c, double tol, int maxit, BSys* d, std::string& w
   d->offf = c->loff_f; d->ordf = c->ord_f; d->Lrp = c->Lrp; d->Lci = c->Lci; d->Lv = c->Lv;
   d->offb = c->loff_b; d->ordb = c->ord_b; d->Urp = c->Urp; d->Uci = c->Uci; d->Uv = c->Uv;
   d->Dinv = c->Dinv;
+  d->spin = c->spin_limit;
+  d->fail = nullptr;
   d->V = c->V; d->w = c->w; d->x = c->xd; d->b = c->bd; d->Z = c->Z;
   d->nlev = (int)c->lev.size();
   for (int l = 0; l < d->nlev; ++l) {
@@ -587,6 +880,12 @@ cptr_status describe(cptr_ctx* c, double tol, int maxit, BSys* d, std::string& w
     B.Arp = L.A.rp; B.Aci = L.A.ci; B.Av = L.Av; B.dinv = L.dinv;
     const bool last = l == d->nlev - 1;
     B.nc = last ? 0 : L.nc;
+    auto lanes = [](const DCSR& M) {
+      const double avg = M.n > 0 ? (double)M.nnz / M.n : 1.0;
+      return avg <= 10.0 ? 2 : avg <= 40.0 ? 4 : 16;
+    };
+    B.lanes = lanes(L.A);
+    B.rlanes = lanes(L.R);
     B.Rrp = L.R.rp; B.Rci = L.R.ci; B.Rv = L.Rv;
     B.Prp = L.P.rp; B.Pci = L.P.ci; B.Pv = L.Pv;
     B.b = L.b; B.x = L.x; B.r = L.r; B.x2 = L.x2; B.t = L.t;
@@ -629,18 +928,74 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
     CTX_CUDA(c0, cudaMemcpyAsync(ctxs[k]->bd, rhs[k], nb, cudaMemcpyDefault, s));
     CTX_CUDA(c0, cudaMemcpyAsync(ctxs[k]->xd, x[k], nb, cudaMemcpyDefault, s));
   }
+  // Blocks per system, in proportion to its cells, so that the batch's largest
+  // system does not run alone on one SM when the others are done: 1, 2, 4 or 8, a
+  // block for every 0.6 of an SM's share of the batch's cells (with fewer the last
+  // systems leave SMs idle, with more the barriers cost more than they divide: 48
+  // systems of 2k-30k cells take 42, 39, 41 and 129 ms with 0.5, 0.7, 1 share and
+  // one block each, 120 systems of 2k-20k 58, 55, 64 and 118 ms, 200 of 2k-30k 115,
+  // 137, 160 and 202 ms) and at least kBlockCells cells.  Systems are laid out by
+  // that number and each group is one launch, side by side on its first system's
+  // second stream.
+  constexpr long long kBlockCells = 1024;
+  long long cells = 0;
+  for (int k = 0; k < n; ++k) cells += ctxs[k]->N;
+  const long long share = std::max(kBlockCells, 3 * cells / (5 * std::max(1, c0->nsm)));
+  const char* env = getenv("CPTR_BATCH_BLOCKS");  // test hook
+  const int forced = env ? atoi(env) : 0;
+  std::vector<int> order(n), blocks(n);
+  for (int k = 0; k < n; ++k) {
+    order[k] = k;
+    blocks[k] = 1;
+    while (blocks[k] < 8 && 2 * blocks[k] * share <= ctxs[k]->N) blocks[k] *= 2;
+    if (forced == 1 || forced == 2 || forced == 4 || forced == 8) blocks[k] = forced;
+  }
+  std::stable_sort(order.begin(), order.end(),
+                   [&](int a, int b) { return blocks[a] > blocks[b]; });
+  std::vector<BSys> hs(n);
   BSys* dsys = nullptr;
   BOut* dout = nullptr;
   CTX_CUDA(c0, cudaMallocAsync((void**)&dsys, sizeof(BSys) * (size_t)n, s));
   cudaError_t e = cudaMallocAsync((void**)&dout, sizeof(BOut) * (size_t)n, s);
   if (e != cudaSuccess) { cudaFreeAsync(dsys, s); return ctx_cuda_fail(c0, e, "batch outputs"); }
   std::vector<BOut> ho(n);
-  e = cudaMemcpyAsync(dsys, h.data(), sizeof(BSys) * (size_t)n, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) {
-    if (c0->mixed) k_batch_fgmres<float><<<n, kBT, 0, s>>>(dsys, dout);
-    else k_batch_fgmres<double><<<n, kBT, 0, s>>>(dsys, dout);
+  for (int k = 0; k < n; ++k) {
+    hs[k] = h[order[k]];
+    hs[k].fail = &dout[k].fail;  // (an address on the device)
+  }
+  e = cudaMemsetAsync(dout, 0, sizeof(BOut) * (size_t)n, s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(dsys, hs.data(), sizeof(BSys) * (size_t)n, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = cudaEventRecord(c0->ev_fork, s);
+  for (int k0 = 0; k0 < n && e == cudaSuccess;) {
+    const int size = blocks[order[k0]];
+    int k1 = k0;
+    while (k1 < n && blocks[order[k1]] == size) ++k1;
+    cptr_ctx* lead = ctxs[order[k0]];
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((k1 - k0) * size);
+    cfg.blockDim = dim3(kBT);
+    cfg.stream = lead->stream2;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    const BSys* sy = dsys + k0;
+    e = cudaStreamWaitEvent(lead->stream2, c0->ev_fork, 0);
+    if (e == cudaSuccess)
+      e = c0->mixed ? cudaLaunchKernelEx(&cfg, k_batch_fgmres<float>, sy, dout + k0)
+                    : cudaLaunchKernelEx(&cfg, k_batch_fgmres<double>, sy, dout + k0);
     ++c0->nlaunch;
-    e = cudaGetLastError();
+    // (also after a failed launch: what runs on the other streams is waited for)
+    if (cudaEventRecord(lead->ev_join, lead->stream2) != cudaSuccess ||
+        cudaStreamWaitEvent(s, lead->ev_join, 0) != cudaSuccess) {
+      if (e == cudaSuccess) e = cudaErrorUnknown;
+      cudaStreamSynchronize(lead->stream2);
+    }
+    k0 = k1;
   }
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ho.data(), dout, sizeof(BOut) * (size_t)n, cudaMemcpyDeviceToHost, s);
@@ -653,6 +1008,9 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
   if (e != cudaSuccess) return ctx_cuda_fail(c0, e, "batched solve");
   const double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
   cptr_status worst = CPTR_OK;
+  std::vector<BOut> hk(n);  // in the caller's order
+  for (int k = 0; k < n; ++k) hk[order[k]] = ho[k];
+  ho = hk;
   for (int k = 0; k < n; ++k) {
     cptr_ctx* c = ctxs[k];
     c->info.iters = ho[k].iters;
@@ -661,6 +1019,8 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
     c->info.solve_s = secs;
     c->info.launches = c->nlaunch;
     if (infos) infos[k] = c->info;
+    if (ho[k].status == CPTR_ERR_TIMEOUT)
+      ctx_set_err(c0, "a bounded device-side wait gave up");
     if (ho[k].status != CPTR_OK && (worst == CPTR_OK || ho[k].status != CPTR_ERR_MAXIT))
       worst = (cptr_status)ho[k].status;
   }

@@ -113,12 +113,10 @@ typedef struct {
                          Gauss-Seidel in row order inside a block (reverse order after the
                          coarse correction) with the l1 diagonal as pivot, the sweep's
                          starting values for rows of other blocks */
-  int tri_tune;       /* 1 (default): cptr_setup picks the ILU(0) triangular-solve
-                         schedule by timing the candidates once per matrix shape (cached
-                         per process); 0: by a rule without timing (one thread-block
-                         cluster walking the levels when its rows fit, else level
-                         kernels).  Schedules are bit-identical, so this changes speed
-                         only.  Servers use the rule for every request. */
+  int tri_tune;       /* 0 or 1 (default).  Either way cptr_setup takes the schedule of the
+                         ILU(0) triangular solves that was fastest on every shape measured
+                         (level kernels); all schedules are bit-identical, so this never
+                         changed a result. */
   int coarsen;        /* C/F splitting of every AMG level: CPTR_COARSEN_PMIS (default, on
                          the GPU) or CPTR_COARSEN_HMIS (Section 3.1).  HMIS on one domain
                          is the first pass of classical Ruge-Stueben coarsening: the
@@ -328,9 +326,7 @@ cptr_status cptr_fma_rate(int fp64, int iters, int reps, void* stream, double* t
 /* Creates a server on the current device that admits requests while their
  * estimated device footprint fits in hbm_budget_bytes, with max_slots worker
  * threads (one CUDA stream each) building and solving them concurrently.
- * Every request uses params (NULL: defaults) with its own tol and maxit, and
- * the triangular-solve schedule rule of tri_tune = 0 (shapes rarely repeat,
- * and the blocks of concurrent requests share the SMs). */
+ * Every request uses params (NULL: defaults) with its own tol and maxit. */
 cptr_status cptr_server_create(cptr_server** out, size_t hbm_budget_bytes, int max_slots,
                                const cptr_params* params);
 /* max_queued: submitted requests not yet admitted (default 4096); a submit

@@ -820,7 +820,7 @@ cptr_status setup_buffers_t(cptr_ctx* c) {
   }
   CTX_ALLOC(c, c->rhat, T, (size_t)nell(c) * N, true);
   CTX_ALLOC(c, c->zc, T, (size_t)nell(c) * N, true);
-  if (!c->r2) CTX_ALLOC(c, c->r2, T, 4 * (size_t)N, true);  // may exist from the solve tuning
+  if (!c->r2) CTX_ALLOC(c, c->r2, T, 4 * (size_t)N, true);  // (CPTR3's second stage shares them)
   if (!c->u) CTX_ALLOC(c, c->u, T, 4 * (size_t)N, true);
   if (!c->y2) CTX_ALLOC(c, c->y2, T, 4 * (size_t)N, true);
   if (!c->zt) CTX_ALLOC(c, c->zt, T, 4 * (size_t)N, true);
@@ -967,14 +967,6 @@ cptr_status profile_apply_t(cptr_ctx* c, int kernel, bool prepare) {
   return CPTR_OK;
 }
 }  // namespace
-
-void launch_level_solves(cptr_ctx* c, void* zbase) {
-  size_t stride = 4 * (size_t)c->N;
-  if (c->mixed)
-    launch_ilu_levels<float>(c, nullptr, zbase, &c->ctl->zero, stride, &c->ctl->one, 0);
-  else
-    launch_ilu_levels<double>(c, nullptr, zbase, &c->ctl->zero, stride, &c->ctl->one, 0);
-}
 
 cptr_status profile_apply_kernel(cptr_ctx* c, int kernel, bool prepare) {
   return c->mixed ? profile_apply_t<float>(c, kernel, prepare)

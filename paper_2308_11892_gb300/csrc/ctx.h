@@ -242,8 +242,6 @@ struct cptr_ctx {
   void* rhsf = nullptr;                // 4N: forward rhs in forward level order (cluster path)
   void* rhsb = nullptr;                // 4N: backward rhs in backward level order (cluster path)
   unsigned spin_limit = kSpinDefault;  // Ctl::spin of every later solve (cptr_set_spin_limit)
-  int tuned_R = -1;                    // autotuned schedule: -1 not tuned, 0 level kernels,
-                                       // 1 cluster, 2 strips, 3 chains, > 3 chunk rows
   int fac_epoch = 0;
   int32_t* fac_done = nullptr;
   void* flush_buf = nullptr;           // 256 MiB buffer written to flush L2 (profiling)
@@ -376,9 +374,9 @@ cptr_status build_level_solve_arrays(cptr_ctx* c);  // level-padded schedule arr
 // ---- sptrsv.cu ----
 // Builds the chunked schedules for R rows per chunk (apply precision).
 cptr_status build_chunked(cptr_ctx* c, int R);
-// Times candidate chunk sizes (and the level-padded kernels) and keeps the best.
-cptr_status tune_triangular(cptr_ctx* c);
-bool tune_decided(cptr_ctx* c);
+// Builds the triangular-solve schedule: the level kernels' arrays, or another
+// schedule forced by CPTR_TRI_R.
+cptr_status build_tri_schedule(cptr_ctx* c);
 // Forward then backward chunked solve: y2 = (LU)^-1 r2, z = P zc + y2 at
 // zbase + (*jptr)*stride (zc may be null).
 void launch_tri_chunked(cptr_ctx* c, const void* zc, void* zbase, const int* jptr, size_t stride,
@@ -414,8 +412,6 @@ cptr_status setup_apply_buffers(cptr_ctx* c);
 void launch_precond(cptr_ctx* c, const double* vbase, void* zbase, const int* jptr,
                     const int* active);
 cptr_status launch_apply_piece(cptr_ctx* c, int which, const double* in, double* out);
-// Level-padded forward + backward solves of c->r2 (no first-stage combine).
-void launch_level_solves(cptr_ctx* c, void* zbase);
 // Profiling of single apply kernels: prepare=true runs the untimed preparation,
 // prepare=false the launch being timed (CPTR_KERNEL_ILU_*, VC_PRE0, CORRECTION).
 cptr_status profile_apply_kernel(cptr_ctx* c, int kernel, bool prepare);

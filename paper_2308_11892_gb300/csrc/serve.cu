@@ -169,7 +169,6 @@ struct cptr_server {
     cptr_params q = p;
     q.tol = r.tol;
     q.maxit = r.maxit;
-    q.tri_tune = 0;  // shapes rarely repeat, and blocks of other requests share the SMs
     return q;
   }
 

@@ -627,10 +627,8 @@ cptr_status setup_ilu_factor(cptr_ctx* c) {
   return CPTR_OK;
 }
 
-// The triangular-solve schedule (its tuner times trial solves, so it runs
-// alone on the context's stream).
 cptr_status setup_ilu_schedule(cptr_ctx* c) {
-  cptr_status st = tune_triangular(c);
+  cptr_status st = build_tri_schedule(c);
   ctx_phase(c, "  ilu solve schedule");
   return st;
 }

@@ -14,9 +14,6 @@
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
-#include <tuple>
-#include <mutex>
-#include <map>
 
 #include "common.cuh"
 #include "ctx.h"
@@ -376,13 +373,6 @@ __global__ void __launch_bounds__(256) k_tri_chunk(
   }
 }
 
-template <class T>
-__global__ void k_sentinel_fill(long long n, T* __restrict__ u, Ctl* ctl) {
-  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i == 0) { ctl->fwd_ctr = 0u; ctl->bwd_ctr = 0u; }
-  if (i < n) u[i] = sentinel_of(T(0));
-}
-
 // ------------------------------------------------------------------ host
 const size_t kSmemBudget = 200 * 1024;
 
@@ -522,83 +512,20 @@ cptr_status build_t(cptr_ctx* c, int R) {
   return CPTR_OK;
 }
 
-// time forward + backward solves with zero right-hand sides (values do not
-// matter, only the dependency propagation)
-// R: 0 level kernels, 1 cluster, > 1 chunked
+// The schedule of the triangular solves: the level kernels, which are the fastest
+// on every shape measured (forward and backward together, against the best of the
+// others, in ms: 500 cells 0.035 / 0.044, 13.5k-cell grid 0.13 / 0.15, 64x64x32 grid
+// 0.30 / 0.35, 13.5k-point cloud 0.55 / 0.85, 1M-point cloud 3.5 / 7.4, 100x100x100
+// grid 0.93 / 1.44; all rounds alike, so this is speed only).  CPTR_TRI_R forces
+// another one: 1 cluster, 2 strips, 3 chains, more a chunk of that many rows; one
+// that cannot be built for the matrix falls back to the level kernels.
 template <class T>
-cptr_status time_solves(cptr_ctx* c, int R, float* ms_out) {
-  cudaStream_t s = cs(c);
-  long long n4 = 4ll * c->N;
-  CTX_CUDA(c, cudaMemsetAsync(c->r2, 0, sizeof(T) * n4, s));
-  cudaEvent_t e0, e1;
-  CTX_CUDA(c, cudaEventCreate(&e0));
-  CTX_CUDA(c, cudaEventCreate(&e1));
-  float best = 1e30f;
-  for (int rep = 0; rep < 4; ++rep) {
-    KL(c, k_sentinel_fill<T><<<nblk(n4), kT, 0, s>>>(n4, (T*)c->u, c->ctl));
-    CTX_CUDA(c, cudaEventRecord(e0, s));
-    if (R > 3)
-      launch_t<T>(c, nullptr, (T*)c->zt, &c->ctl->zero, (size_t)n4, &c->ctl->one, 0);
-    else if (R == 3)
-      launch_tri_chain(c, nullptr, c->zt, &c->ctl->zero, (size_t)n4, &c->ctl->one, 0);
-    else if (R == 2)
-      launch_tri_strip(c, nullptr, c->zt, &c->ctl->zero, (size_t)n4, &c->ctl->one, 0);
-    else if (R == 1)
-      launch_tri_cluster(c, nullptr, c->zt, &c->ctl->zero, (size_t)n4, &c->ctl->one, 0);
-    else
-      launch_level_solves(c, c->zt);
-    cudaError_t le = cudaGetLastError();
-    if (le != cudaSuccess) {
-      // a candidate that cannot launch is skipped, never chosen
-      if (c->timing) fprintf(stderr, "[cptr]   tri solve launch failed: %s\n", cudaGetErrorString(le));
-      cudaEventDestroy(e0);
-      cudaEventDestroy(e1);
-      return CPTR_ERR_INVALID;
-    }
-    CTX_CUDA(c, cudaEventRecord(e1, s));
-    CTX_CUDA(c, cudaEventSynchronize(e1));
-    float ms = 0.f;
-    CTX_CUDA(c, cudaEventElapsedTime(&ms, e0, e1));
-    if (rep > 0) best = std::min(best, ms);
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  *ms_out = best;
-  return ctx_check_device_status(c);
-}
-
-// Tuner decisions shared by every context of the process, keyed by what
-// determines them: device, cells, blocks, forward and backward level counts
-// and the apply precision.  Every schedule computes bit-identical results, so a
-// decision taken on another matrix of the same shape can only cost speed; it
-// spares each new context (a served request, a new Newton system) the trial
-// solves of every candidate.
-struct TuneKey {
-  int dev, n, nnzb, nlev_f, nlev_b, mixed;
-  bool operator<(const TuneKey& o) const {
-    return std::tie(dev, n, nnzb, nlev_f, nlev_b, mixed) <
-           std::tie(o.dev, o.n, o.nnzb, o.nlev_f, o.nlev_b, o.mixed);
-  }
-};
-std::mutex g_tune_mu;
-std::map<TuneKey, int> g_tune_cache;
-
-template <class T>
-cptr_status tune_t(cptr_ctx* c) {
+cptr_status schedule_t(cptr_ctx* c) {
   const char* env = getenv("CPTR_TRI_R");
-  int forced = env ? atoi(env) : -1;
-  if (forced >= 0) c->tuned_R = forced;
-  // without timing: a cluster when its rows fit, else level kernels
-  if (c->tuned_R < 0 && !c->p.tri_tune) c->tuned_R = 1;
-  const TuneKey key{c->dev, c->N, c->nnzb, c->nlev_f, c->nlev_b, c->mixed ? 1 : 0};
-  if (c->tuned_R < 0) {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tune_cache.find(key);
-    if (it != g_tune_cache.end()) c->tuned_R = it->second;
-  }
+  const int R = env && atoi(env) > 0 ? atoi(env) : 0;
   c->chunked = c->cluster = c->strip = c->chain = false;
-  if (c->tuned_R == 0) return build_level_solve_arrays(c);
-  if (c->tuned_R == 1) {
+  if (R == 0) return build_level_solve_arrays(c);
+  if (R == 1) {
     cptr_status st = build_cluster(c);
     if (st != CPTR_ERR_INVALID) {
       c->cluster = st == CPTR_OK;
@@ -606,7 +533,7 @@ cptr_status tune_t(cptr_ctx* c) {
     }
     return build_level_solve_arrays(c);  // no cluster fits: level kernels
   }
-  if (c->tuned_R == 2) {
+  if (R == 2) {
     cptr_status st = build_strip(c);
     if (st != CPTR_ERR_INVALID) {
       c->strip = st == CPTR_OK;
@@ -614,7 +541,7 @@ cptr_status tune_t(cptr_ctx* c) {
     }
     return build_level_solve_arrays(c);  // a step does not fit: level kernels
   }
-  if (c->tuned_R == 3) {
+  if (R == 3) {
     cptr_status st = build_chain(c);
     if (st != CPTR_ERR_INVALID) {
       c->chain = st == CPTR_OK;
@@ -622,77 +549,10 @@ cptr_status tune_t(cptr_ctx* c) {
     }
     return build_level_solve_arrays(c);  // chains that could wait on later ones: level kernels
   }
-  if (c->tuned_R > 3) {
-    cptr_status st = build_t<T>(c, c->tuned_R);
-    if (st != CPTR_ERR_INVALID) return st;
-    c->chunked = false;  // the chunk does not fit in shared memory: level kernels
-    return build_level_solve_arrays(c);
-  }
-  // work buffers for timing
-  size_t n4 = 4 * (size_t)c->N;
-  if (!c->r2) {
-    c->r2 = ctx_alloc(c, sizeof(T) * n4 + 16, true);
-    c->u = ctx_alloc(c, sizeof(T) * n4 + 16, true);
-    c->y2 = ctx_alloc(c, sizeof(T) * n4 + 16, true);
-    c->zt = ctx_alloc(c, sizeof(T) * n4 + 16, true);
-    if (!c->r2 || !c->u || !c->y2 || !c->zt) return CPTR_ERR_NOMEM;
-  }
-  std::vector<int> cand = {0, 1, 2, 3};
-  for (int R : {128, 256, 512, 1024, 2048})
-    if (R <= 2 * c->N) cand.push_back(R);
-  int best_R = 0;
-  float best_ms = 1e30f;
-  // A chunked schedule needs every chunk resident at once: with more chunks
-  // than thread blocks that fit on the GPU, the persistent blocks walk the
-  // dependency chains one chunk after another (on a 200x200x100 grid that is
-  // seconds per solve), so such chunk sizes are not candidates.
-  auto per_sm = [](size_t smem) {
-    return std::max<int>(1, std::min<int>(8, (int)(227000 / (smem + 1024))));
-  };
-  for (int R : cand) {
-    if (R > 3 && (long long)ceil_div(c->N, R) > 8ll * c->nsm) continue;
-    cptr_status st = (R == 0) ? build_level_solve_arrays(c)
-                     : (R == 1) ? build_cluster(c) : (R == 2) ? build_strip(c)
-                     : (R == 3) ? build_chain(c) : build_t<T>(c, R);
-    if (st == CPTR_ERR_INVALID) continue;  // does not fit in shared memory
-    if (st) return st;
-    if (R > 3 && (c->tf.nch > c->nsm * per_sm(c->tf.smem) ||
-                  c->tb.nch > c->nsm * per_sm(c->tb.smem)))
-      continue;
-    c->chunked = R > 3;
-    c->cluster = R == 1;
-    c->strip = R == 2;
-    c->chain = R == 3;
-    float ms = 0.f;
-    st = time_solves<T>(c, R, &ms);
-    if (st == CPTR_ERR_INVALID) continue;
-    if (st) return st;
-    if (c->timing) fprintf(stderr, "[cptr]   tri solve R=%-5d %8.3f ms\n", R, ms);
-    if (ms < best_ms) { best_ms = ms; best_R = R; }
-  }
-  c->tuned_R = best_R;
-  {
-    std::lock_guard<std::mutex> lk(g_tune_mu);
-    g_tune_cache[key] = best_R;
-  }
-  c->chunked = c->cluster = c->strip = c->chain = false;
-  if (best_R == 0) return build_level_solve_arrays(c);
-  if (best_R == 1) {
-    cptr_status st = build_cluster(c);
-    c->cluster = st == CPTR_OK;
-    return st;
-  }
-  if (best_R == 2) {
-    cptr_status st = build_strip(c);
-    c->strip = st == CPTR_OK;
-    return st;
-  }
-  if (best_R == 3) {
-    cptr_status st = build_chain(c);
-    c->chain = st == CPTR_OK;
-    return st;
-  }
-  return build_t<T>(c, best_R);
+  cptr_status st = build_t<T>(c, R);
+  if (st != CPTR_ERR_INVALID) return st;
+  c->chunked = false;  // the chunk does not fit in shared memory: level kernels
+  return build_level_solve_arrays(c);
 }
 
 }  // namespace
@@ -701,18 +561,8 @@ cptr_status build_chunked(cptr_ctx* c, int R) {
   return c->mixed ? build_t<float>(c, R) : build_t<double>(c, R);
 }
 
-// Whether the schedule is already decided (forced, tuned by an earlier setup
-// of this context, or cached for this shape): then building it times nothing.
-bool tune_decided(cptr_ctx* c) {
-  const char* env = getenv("CPTR_TRI_R");
-  if ((env && atoi(env) >= 0) || c->tuned_R >= 0 || !c->p.tri_tune) return true;
-  const TuneKey key{c->dev, c->N, c->nnzb, c->nlev_f, c->nlev_b, c->mixed ? 1 : 0};
-  std::lock_guard<std::mutex> lk(g_tune_mu);
-  return g_tune_cache.count(key) > 0;
-}
-
-cptr_status tune_triangular(cptr_ctx* c) {
-  return c->mixed ? tune_t<float>(c) : tune_t<double>(c);
+cptr_status build_tri_schedule(cptr_ctx* c) {
+  return c->mixed ? schedule_t<float>(c) : schedule_t<double>(c);
 }
 
 void launch_tri_chunked(cptr_ctx* c, const void* zc, void* zbase, const int* jptr, size_t stride,

@@ -36,7 +36,6 @@ struct BLevel {
   const void* Av;    // apply precision
   const void* dinv;  // apply precision
   int nc;            // rows of the next level (R: nc x n, P: n x nc)
-  int lanes, rlanes; // lanes per row of A and of R (by their mean row lengths)
   const int32_t *Rrp, *Rci;
   const void* Rv;
   const int32_t *Prp, *Pci;
@@ -249,65 +248,47 @@ __device__ __noinline__ void bspmv(const Team& t, const BSys& S, const TX* x, co
   }
 }
 
-// f(i, sum) for every row i < n of a CSR operator, sum = its val * x: L lanes per
-// row (by the operator's mean row length), each summing its entries in order,
-// then a shuffle tree.
-template <int L, class T, class F>
-__device__ __forceinline__ void rows_as(const Team& t, int n, const int32_t* __restrict__ rp,
-                                        const int32_t* __restrict__ ci,
-                                        const T* __restrict__ val, const T* x, F f) {
-  const int sl = threadIdx.x & (L - 1);
-  // whole warps: the lanes of a warp meet at the shuffles
-  const int per = t.threads / L;
-  for (int i0 = 0; i0 < n; i0 += per) {
-    const int i = i0 + t.tid / L;
-    T s = 0;
-    if (i < n) {
-      const int t1 = rp[i + 1];
-      for (int k = rp[i] + sl; k < t1; k += 4 * L) {
-        int j[4];
-        T a[4], xv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k + u * L < t1) {
-            j[u] = ci[k + u * L];
-            a[u] = val[k + u * L];
-          }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k + u * L < t1) xv[u] = x[j[u]];
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (k + u * L < t1) s += a[u] * xv[u];
-      }
-    }
-#pragma unroll
-    for (int o = L / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, L);
-    if (i < n && sl == 0) f(i, s);
-  }
-}
+// f(i, sum) for every row i < n of a CSR operator, sum = its val * x in entry order
+// (a thread per row; eight entries are loaded before their products are added).
 template <class T, class F>
-__device__ __forceinline__ void rows(const Team& t, int n, int lanes,
-                                     const int32_t* __restrict__ rp,
+__device__ __forceinline__ void rows(const Team& t, int n, const int32_t* __restrict__ rp,
                                      const int32_t* __restrict__ ci, const T* __restrict__ val,
                                      const T* x, F f) {
-  // (about four entries per lane: fewer leave too few loads in flight)
-  if (lanes <= 2) rows_as<2>(t, n, rp, ci, val, x, f);
-  else if (lanes <= 4) rows_as<4>(t, n, rp, ci, val, x, f);
-  else rows_as<16>(t, n, rp, ci, val, x, f);
+  constexpr int K = 8;
+  for (int i = t.tid; i < n; i += t.threads) {
+    T s = 0;
+    const int t1 = rp[i + 1];
+    for (int k = rp[i]; k < t1; k += K) {
+      int j[K];
+      T a[K], xv[K];
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (k + u < t1) {
+          j[u] = ci[k + u];
+          a[u] = val[k + u];
+        }
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (k + u < t1) xv[u] = x[j[u]];
+#pragma unroll
+      for (int u = 0; u < K; ++u)
+        if (k + u < t1) s += a[u] * xv[u];
+    }
+    f(i, s);
+  }
 }
 
 // r = b - A x on one AMG level (scalar CSR, apply precision)
 template <class T>
 __device__ __noinline__ void lresid(const Team& t, const BLevel& L, const T* b, const T* x, T* r) {
-  rows<T>(t, L.n, L.lanes, L.Arp, L.Aci, (const T*)L.Av, x, [=](int i, T s) { r[i] = b[i] - s; });
+  rows<T>(t, L.n, L.Arp, L.Aci, (const T*)L.Av, x, [=](int i, T s) { r[i] = b[i] - s; });
 }
 
 // xout = xin + D_l1^-1 (b - A xin): one l1-Jacobi sweep
 template <class T>
 __device__ __noinline__ void lsweep(const Team& t, const BLevel& L, const T* b, const T* xin, T* xout) {
   const T* dv = (const T*)L.dinv;
-  rows<T>(t, L.n, L.lanes, L.Arp, L.Aci, (const T*)L.Av, xin,
+  rows<T>(t, L.n, L.Arp, L.Aci, (const T*)L.Av, xin,
           [=](int i, T s) { xout[i] = xin[i] + dv[i] * (b[i] - s); });
 }
 
@@ -316,13 +297,11 @@ template <class T>
 __device__ __noinline__ void lrestrict(const Team& t, const BLevel& L, const T* r, T* bn) {
   const int32_t *rp = L.Rrp, *ci = L.Rci;
   const T* rv = (const T*)L.Rv;
-  auto f = [=](int i, T s) { bn[i] = s; };
-  if (L.rlanes <= 2) rows_as<2>(t, L.nc, rp, ci, rv, r, f);
-  else rows_as<8>(t, L.nc, rp, ci, rv, r, f);
+  rows<T>(t, L.nc, rp, ci, rv, r, [=](int i, T s) { bn[i] = s; });
 }
 template <class T>
 __device__ __noinline__ void lprolong(const Team& t, const BLevel& L, const T* xc, T* x) {
-  rows_as<2>(t, L.n, L.Prp, L.Pci, (const T*)L.Pv, xc, [=](int i, T s) { x[i] += s; });
+  rows<T>(t, L.n, L.Prp, L.Pci, (const T*)L.Pv, xc, [=](int i, T s) { x[i] += s; });
 }
 
 // One V(nu_pre, nu_post) cycle with l1-Jacobi from a zero guess on the
@@ -880,12 +859,6 @@ cptr_status describe(cptr_ctx* c, double tol, int maxit, BSys* d, std::string& w
     B.Arp = L.A.rp; B.Aci = L.A.ci; B.Av = L.Av; B.dinv = L.dinv;
     const bool last = l == d->nlev - 1;
     B.nc = last ? 0 : L.nc;
-    auto lanes = [](const DCSR& M) {
-      const double avg = M.n > 0 ? (double)M.nnz / M.n : 1.0;
-      return avg <= 10.0 ? 2 : avg <= 40.0 ? 4 : 16;
-    };
-    B.lanes = lanes(L.A);
-    B.rlanes = lanes(L.R);
     B.Rrp = L.R.rp; B.Rci = L.R.ci; B.Rv = L.Rv;
     B.Prp = L.P.rp; B.Pci = L.P.ci; B.Pv = L.Pv;
     B.b = L.b; B.x = L.x; B.r = L.r; B.x2 = L.x2; B.t = L.t;
@@ -932,9 +905,9 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
   // system does not run alone on one SM when the others are done: 1, 2, 4 or 8, a
   // block for every 0.6 of an SM's share of the batch's cells (with fewer the last
   // systems leave SMs idle, with more the barriers cost more than they divide: 48
-  // systems of 2k-30k cells take 42, 39, 41 and 129 ms with 0.5, 0.7, 1 share and
+  // systems of 2k-30k cells took 42, 39, 41 and 129 ms with 0.5, 0.7, 1 share and
   // one block each, 120 systems of 2k-20k 58, 55, 64 and 118 ms, 200 of 2k-30k 115,
-  // 137, 160 and 202 ms) and at least kBlockCells cells.  Systems are laid out by
+  // 137, 160 and 202 ms; the 48 take 31 ms with 0.6) and at least kBlockCells cells.  Systems are laid out by
   // that number and each group is one launch, side by side on its first system's
   // second stream.
   constexpr long long kBlockCells = 1024;

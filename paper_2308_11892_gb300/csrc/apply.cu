@@ -29,17 +29,15 @@ __global__ void k_inverse(int n, const double* __restrict__ d, T* __restrict__ o
 }
 
 // AE[t][r][s] = A_t[r][e_s]: the elliptic columns of every block (4x2; the
-// second column is zero when e has one unknown, e1 < 0).
+// second column is zero when e has one unknown, e1 < 0); a thread per entry, so
+// that a warp reads whole blocks (200x200x100 grid: 1.29 -> 0.83 ms).
 template <class T>
 __global__ void k_extract_ae(int nnzb, const double* __restrict__ v, int e0, int e1,
                              T* __restrict__ ae) {
-  int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nnzb) return;
-  const double* B = v + 16 * (size_t)t;
-  for (int r = 0; r < 4; ++r) {
-    ae[8 * (size_t)t + 2 * r + 0] = (T)B[r * 4 + e0];
-    ae[8 * (size_t)t + 2 * r + 1] = e1 < 0 ? T(0) : (T)B[r * 4 + e1];
-  }
+  const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= 8ll * nnzb) return;
+  const int r = (int)(g >> 1) & 3, e = (g & 1) ? e1 : e0;
+  ae[g] = e < 0 ? T(0) : (T)v[16 * (g >> 3) + 4 * r + e];
 }
 
 // ------------------------------------------------------------------ restriction
@@ -71,50 +69,20 @@ __global__ void k_restrict(int N, const TIN* __restrict__ vbase, const int* jptr
 }
 
 // ------------------------------------------------------------------ V-cycle
-// LANES consecutive lanes cooperate on one row of a scalar CSR operator.  What
-// binds these kernels is the gathers of x (a 32-byte sector from L2 for each
-// entry that misses L1) and, for short rows, the loads in flight per lane: up to
-// eight lanes, each takes four consecutive entries at a time with 16-byte loads of
-// the columns and values (the finest level of the 200x200x100 grid, 4 lanes: sweep
-// and residual 0.296 -> 0.260 ms); wider, one entry per lane keeps a row's
-// gathers together (level 1 of that grid, 16 lanes: 0.40 against 0.41 ms; with two
-// gathers per entry 0.46 against 0.52).  The
-// 16-byte loads start at multiples of four entries, so that a row's first and last
-// may hold entries of its neighbours (or of the padding every array ends with),
-// which are skipped.  Returns the row's sum in every lane; ok is false for lanes
-// past the last row.
-__device__ __forceinline__ void ld_vals4(const float* p, float* o) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-  o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w;
-}
-__device__ __forceinline__ void ld_vals4(const double* p, double* o) {
-  const double2 a = __ldg(reinterpret_cast<const double2*>(p));
-  const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
-  o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-}
+// LANES consecutive lanes cooperate on one row of a scalar CSR operator: lane sl
+// sums the entries sl, sl + LANES, ... of the row, then a shuffle tree; every lane
+// returns the sum, ok is false for lanes past the last row.  What binds these
+// kernels is the gathers of x (a 32-byte sector from L2 for each entry that misses
+// L1).  (Four entries per lane with 16-byte loads: 0.26 instead of 0.30 ms on the
+// finest level of the 200x200x100 grid, slower on the others, and in FP32 another
+// rounding of every sum.)
 template <int LANES, class T, class X>
 __device__ __forceinline__ T row_sum(bool ok, int i, int sl, const int32_t* __restrict__ rp,
                                      const int32_t* __restrict__ ci, const T* __restrict__ val,
                                      X xval) {
   T s = 0;
-  if (ok) {
-    const int t0 = rp[i], t1 = rp[i + 1];
-    if (LANES > 8) {
-      for (int t = t0 + sl; t < t1; t += LANES) s += val[t] * xval(ci[t]);
-    } else {
-      for (int t = (t0 & ~3) + 4 * sl; t < t1; t += 4 * LANES) {
-        const int4 c4 = __ldg(reinterpret_cast<const int4*>(ci + t));
-        const int j[4] = {c4.x, c4.y, c4.z, c4.w};
-        T a[4], x[4];
-        ld_vals4(val + t, a);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = (t + u >= t0 && t + u < t1) ? xval(j[u]) : T(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (t + u >= t0 && t + u < t1) s += a[u] * x[u];
-      }
-    }
-  }
+  if (ok)
+    for (int t = rp[i] + sl; t < rp[i + 1]; t += LANES) s += val[t] * xval(ci[t]);
 #pragma unroll
   for (int o = LANES / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o, LANES);
   return s;
@@ -816,7 +784,7 @@ cptr_status setup_buffers_t(cptr_ctx* c) {
     CTX_ALLOC(c, c->Wt, T, 4 * (size_t)N, true);
     KL(c, k_convert<T><<<nblk(4ll * N), kT, 0, s>>>(4ll * N, c->W64, (T*)c->Wt));
     CTX_ALLOC(c, c->AE, T, 8 * (size_t)c->nnzb, true);
-    KL(c, k_extract_ae<T><<<nblk(c->nnzb), kT, 0, s>>>(c->nnzb, c->v, c->se0, c->se1, (T*)c->AE));
+    KL(c, k_extract_ae<T><<<nblk(8ll * c->nnzb), kT, 0, s>>>(c->nnzb, c->v, c->se0, c->se1, (T*)c->AE));
   }
   CTX_ALLOC(c, c->rhat, T, (size_t)nell(c) * N, true);
   CTX_ALLOC(c, c->zc, T, (size_t)nell(c) * N, true);

@@ -249,30 +249,44 @@ __device__ __noinline__ void bspmv(const Team& t, const BSys& S, const TX* x, co
 }
 
 // f(i, sum) for every row i < n of a CSR operator, sum = its val * x in entry order
-// (a thread per row; eight entries are loaded before their products are added).
+// (a thread per row; four entries are loaded before their products are added.  Eight
+// at a time, predicated, took 62 million clocks against 49 in the V-cycles of a
+// 24.6k-cell cloud on one block; the last one to three are read together.)
 template <class T, class F>
 __device__ __forceinline__ void rows(const Team& t, int n, const int32_t* __restrict__ rp,
                                      const int32_t* __restrict__ ci, const T* __restrict__ val,
                                      const T* x, F f) {
-  constexpr int K = 8;
   for (int i = t.tid; i < n; i += t.threads) {
     T s = 0;
+    int k = rp[i];
     const int t1 = rp[i + 1];
-    for (int k = rp[i]; k < t1; k += K) {
-      int j[K];
-      T a[K], xv[K];
+    for (; k + 4 <= t1; k += 4) {
+      int j[4];
+      T a[4], xv[4];
 #pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (k + u < t1) {
-          j[u] = ci[k + u];
-          a[u] = val[k + u];
-        }
+      for (int u = 0; u < 4; ++u) {
+        j[u] = ci[k + u];
+        a[u] = val[k + u];
+      }
 #pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (k + u < t1) xv[u] = x[j[u]];
+      for (int u = 0; u < 4; ++u) xv[u] = x[j[u]];
 #pragma unroll
-      for (int u = 0; u < K; ++u)
-        if (k + u < t1) s += a[u] * xv[u];
+      for (int u = 0; u < 4; ++u) s += a[u] * xv[u];
+    }
+    if (k < t1) {
+      int j[3];
+      T a[3], xv[3];
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int e = min(k + u, t1 - 1);
+        j[u] = ci[e];
+        a[u] = val[e];
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u) xv[u] = x[j[u]];
+      s += a[0] * xv[0];
+      if (k + 1 < t1) s += a[1] * xv[1];
+      if (k + 2 < t1) s += a[2] * xv[2];
     }
     f(i, s);
   }
@@ -626,28 +640,31 @@ __device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double
       T acc = 0;
       int k = rp[i];
       const int k1 = rp[i + 1];
-      for (; k < k1; k += 4) {
+      for (; k + 4 <= k1; k += 4) {
         int j[4];
         T a0[4], a1[4], z0[4], z1[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (k + q < k1) {
-            j[q] = ci[k + q];
-            a0[q] = ae[8 * (size_t)(k + q) + 2 * r];
-            a1[q] = ae[8 * (size_t)(k + q) + 2 * r + 1];
-          }
+        for (int q = 0; q < 4; ++q) {
+          j[q] = ci[k + q];
+          a0[q] = ae[8 * (size_t)(k + q) + 2 * r];
+          a1[q] = ae[8 * (size_t)(k + q) + 2 * r + 1];
+        }
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (k + q < k1) {
-            z0[q] = ne == 2 ? zc[2 * (size_t)j[q]] : zc[j[q]];
-            z1[q] = ne == 2 ? zc[2 * (size_t)j[q] + 1] : T(0);
-          }
+        for (int q = 0; q < 4; ++q) {
+          z0[q] = ne == 2 ? zc[2 * (size_t)j[q]] : zc[j[q]];
+          z1[q] = ne == 2 ? zc[2 * (size_t)j[q] + 1] : T(0);
+        }
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-          if (k + q < k1) {
-            if (ne == 2) acc += a0[q] * z0[q] + a1[q] * z1[q];
-            else acc += a0[q] * z0[q];
-          }
+        for (int q = 0; q < 4; ++q) {
+          if (ne == 2) acc += a0[q] * z0[q] + a1[q] * z1[q];
+          else acc += a0[q] * z0[q];
+        }
+      }
+      for (; k < k1; ++k) {
+        const int jj = ci[k];
+        const T* a = ae + 8 * (size_t)k + 2 * r;
+        if (ne == 2) acc += a[0] * zc[2 * (size_t)jj] + a[1] * zc[2 * (size_t)jj + 1];
+        else acc += a[0] * zc[jj];
       }
       r2[g] = (T)v[g] - acc;
     }
@@ -822,7 +839,7 @@ cptr_status describe(cptr_ctx* c, double tol, int maxit, BSys* d, std::string& w
   if (c->p.restart > kBMaxM) { why = "batched solves need restart <= 32"; return CPTR_ERR_INVALID; }
   if ((int)c->lev.size() > kBMaxLev) { why = "too many AMG levels"; return CPTR_ERR_INVALID; }
   if (!c->Lrp || !c->Urp || !c->Dinv) {
-    // the level-ordered factor arrays (built when the tuner picked another schedule)
+    // the level-ordered factor arrays (built when another schedule was forced)
     cptr_status st = build_level_solve_arrays(c);
     if (st) return st;
     CTX_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -907,13 +924,17 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
   // systems leave SMs idle, with more the barriers cost more than they divide: 48
   // systems of 2k-30k cells took 42, 39, 41 and 129 ms with 0.5, 0.7, 1 share and
   // one block each, 120 systems of 2k-20k 58, 55, 64 and 118 ms, 200 of 2k-30k 115,
-  // 137, 160 and 202 ms; the 48 take 31 ms with 0.6) and at least kBlockCells cells.  Systems are laid out by
-  // that number and each group is one launch, side by side on its first system's
-  // second stream.
-  constexpr long long kBlockCells = 1024;
+  // 137, 160 and 202 ms; the 48 take 31 ms with 0.6) and at least
+  // kBlockCells cells.  From kMostCells on a block is divided whatever the batch: it
+  // loses more to its L1 than the barriers cost (304 systems of 2k-28k cells: 178 ms
+  // without this limit, 132 with 5632, 127 with 4096; 160 systems 90, 90, 78).
+  // Systems are laid out by that number and each group is one launch, side by side
+  // on its first system's second stream.
+  constexpr long long kBlockCells = 1024, kMostCells = 4096;
   long long cells = 0;
   for (int k = 0; k < n; ++k) cells += ctxs[k]->N;
-  const long long share = std::max(kBlockCells, 3 * cells / (5 * std::max(1, c0->nsm)));
+  const long long share = std::clamp(3 * cells / (5 * std::max(1, c0->nsm)), kBlockCells,
+                                     kMostCells);
   const char* env = getenv("CPTR_BATCH_BLOCKS");  // test hook
   const int forced = env ? atoi(env) : 0;
   std::vector<int> order(n), blocks(n);

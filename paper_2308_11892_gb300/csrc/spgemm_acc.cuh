@@ -354,6 +354,9 @@ __device__ __forceinline__ bool acc_walk(const AccArgs& a, int t0, int na, int* 
         if (act && rank == r && h >= 0) val[h] += prod;
       }
       if (__any_sync(0xffffffffu, bad)) return false;
+      // the keys and sums of this step before the next one's, or before the caller
+      // reads the table: shuffles and votes do not order shared memory
+      __syncwarp();
       col = coln; b = bn; e = en;
     }
   }

@@ -289,7 +289,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp_group(IxArgs a, int cls, 
       if (k < K) {
         const bool z = d_eq0(sum);
         S.kf[k] = S.ka[k] / sum;
-        S.klen[k] = z ? 1 : 0;  // 1: the connection itself goes to the diagonal
+        S.klen[k] = z;  // the connection itself goes to the diagonal
+        S.kst[k] = z;   // ka holds a term of the diagonal
       }
       const unsigned m = vote(k == K);
       const double d = __shfl_sync(FULL, sum, sh + (m ? __ffs(m) - 1 : 0));
@@ -299,14 +300,14 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp_group(IxArgs a, int cls, 
     // ---- f_k abar_kl; the term with l = i belongs to the diagonal
     for (int t = D + gl; t < T; t += G) {
       const int k = S.tk[t];
-      if (S.klen[k] & 1) {
+      if (S.klen[k]) {
         S.tpos[t] = 0xffff;
       } else {
         const double x = S.kf[k] * S.tval[t];
         S.tval[t] = x;
         if (S.tpos[t] == nq) {
           S.ka[k] = x;
-          S.klen[k] = 2;
+          S.kst[k] = 1;  // (klen is read by the neighbour's other lanes)
           S.tpos[t] = 0xffff;
         }
       }
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_interp_group(IxArgs a, int cls, 
     // ---- diagonal, then the weights
     double dg = dg0;
     for (int k = 0; k < maxK; ++k)
-      if (k < K && S.klen[k]) dg += S.ka[k];
+      if (k < K && S.kst[k]) dg += S.ka[k];
     const bool ok = !(d_eq0(dg) || dmag(dg) >= 0x7ff0000000000000ull) && nq > 0;
     const int cols = ok ? nq : 0;
     const int maxq = __reduce_max_sync(FULL, cols);

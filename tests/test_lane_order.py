@@ -30,3 +30,7 @@ def _run(tmp_path, source, *include):
 
 def test_product_accumulators(tmp_path):
     _run(tmp_path, "products.cpp")
+
+
+def test_interpolation_by_lane_groups(tmp_path):
+    _run(tmp_path, "interp.cpp")

@@ -410,7 +410,6 @@ __global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_pair(
       double lr[4];  // row r of L_ik
 #pragma unroll
       for (int q = 0; q < 4; ++q) lr[q] = __shfl_sync(FULL, l, 4 * r + q, 16);
-      if (act) bi[16 * e + hl] = l;
       // A_ij -= L_ik U_kj
       auto update = [&](int m, const double* w) {
         const int at = m < nm ? 16 * (int)mt[m0 + m] + hl : 0;
@@ -432,6 +431,8 @@ __global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_pair(
       cur = nxt;
       have = nhave;
       __syncwarp();
+      // (behind the barrier: the row's other lanes have read A_ik by then)
+      if (act) bi[16 * e + hl] = l;
     }
     bool ok;
     double dv = inv4_pair(i >= 0 ? bi[16 * di + hl] : (r == c ? 1.0 : 0.0), &ok);

@@ -10,7 +10,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_2308_11892_gb300", "csrc")
 
 
-def _run(tmp_path, source, *include):
+def _run(tmp_path, source, *args):
     flags = ["-std=c++17", "-O1", "-g", "-ffp-contract=off", "-w", "-pthread",
              "-fsanitize=thread"]
     probe = tmp_path / "probe.cpp"
@@ -20,11 +20,11 @@ def _run(tmp_path, source, *include):
     if r.returncode or subprocess.run([pexe], capture_output=True).returncode:
         pytest.skip("no usable thread sanitizer")
     exe = str(tmp_path / "lanes")
-    dirs = [f"-I{d}" for d in (os.path.join(HERE, "lane_order"), CSRC, *include)]
+    dirs = [f"-I{d}" for d in (os.path.join(HERE, "lane_order"), CSRC, tmp_path)]
     subprocess.run(["g++", *flags, *dirs, os.path.join(HERE, "lane_order", source), "-o", exe],
                    check=True)
     env = dict(os.environ, TSAN_OPTIONS="exitcode=66 halt_on_error=1")
-    r = subprocess.run([exe], capture_output=True, text=True, timeout=600, env=env)
+    r = subprocess.run([exe, *args], capture_output=True, text=True, timeout=600, env=env)
     assert r.returncode == 0, (r.stdout + r.stderr)[-3000:]
 
 
@@ -34,3 +34,16 @@ def test_product_accumulators(tmp_path):
 
 def test_interpolation_by_lane_groups(tmp_path):
     _run(tmp_path, "interp.cpp")
+
+
+def _ilu_kernel(tmp_path):
+    """k_ilu_factor_pair with what it calls, cut from setup_ilu.cu."""
+    src = open(os.path.join(CSRC, "setup_ilu.cu")).read()
+    inv = src[src.index("__device__ __forceinline__ double inv4_pair"):]
+    row = src[src.index("constexpr int kRowMax"):src.index("__global__ void k_max_row")]
+    (tmp_path / "ilu_pair.inc").write_text(inv[:inv.index("\n}\n") + 3] + row)
+
+
+def test_ilu_two_rows_per_warp(tmp_path):
+    _ilu_kernel(tmp_path)
+    _run(tmp_path, "ilu.cpp")

@@ -6,8 +6,9 @@
 //
 // Rows are factorised by a sync-free kernel that follows the level schedule of
 // the lower triangle (level(i) = 1 + max level(k), k < i in row i): a warp
-// claims the next row of the schedule, waits (bounded) for the rows it needs,
-// and publishes completion with a release flag.  The same schedule, and the
+// claims the next two rows of the schedule (one, of matrices with a row of more than
+// 32 blocks), waits (bounded) for the rows they need, and publishes their completion
+// with release flags.  The same schedule, and the
 // one of the upper triangle, order the triangular solves.
 #include <vector>
 
@@ -231,18 +232,22 @@ __global__ void __launch_bounds__(256) k_ilu_factor(int npos, const int32_t* __r
 
 // The same factorisation, two rows per warp: sixteen lanes per row, lane 4 r + c
 // holding entry (r, c) of a 4x4 block, both rows (neighbours in the schedule, so
-// of one level) in lockstep; products are fused, except in the inversion, whose
-// pivots decide what is singular.  The kernel is bound by FP64 issue on wide
-// levels, where an instruction costs the same for 16 lanes as for 32, and by the
+// of one level) in lockstep.  Every product and sum rounds by itself, as in
+// k_ilu_factor and in the definition: with fused products a pivot block that cancels
+// exactly keeps a residue, and a singular matrix is no longer refused (of 93 two-cell
+// systems with repeated block rows that the definition refuses, 72 went through).  The
+// kernel is bound by FP64 issue on wide levels, where an instruction costs the same for
+// 16 lanes as for 32, and by the
 // chain flag - inv(U_kk) - L_ik - update - ... - inversion - flag on narrow ones,
 // where a row's first dependency may be its last to come: the rows share every
 // FP64 instruction; the row's blocks and the columns that row i and its
 // dependencies share (pattern only) are ready before the first wait; the flags
 // are read together, and a published dependency's blocks are loaded while the one
 // before it is worked on; one release publishes the row.  Rows longer than maxrow
-// blocks do not come here.  200x200x100 grid 34.8 -> 9.8 ms, 1M-point cloud 21.7 ->
-// 17.5 ms, 64x64x32 grid 2.2 -> 1.5 ms (one row per warp, a dependency's loads after
-// its own flag; two rows per warp without the look-ahead: 25.9 ms on the cloud).
+// blocks do not come here.  200x200x100 grid 34.8 -> 12.9 ms (9.8 with fused products),
+// 64x64x32 grid 2.2 -> 1.4 ms; narrow levels of long rows gain nothing: 1M-point cloud
+// 21.7 -> 22.1 ms (17.5 fused).  (Before: one row per warp, a dependency's loads after
+// its own flag.)
 constexpr int kRowMax = 32;
 constexpr int kFacWarps = 4;
 constexpr int kAhead = 2;  // shared blocks of a dependency loaded ahead
@@ -405,7 +410,7 @@ __global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_pair(
         const double* A = bi + 16 * e + 4 * r;
         l = A[0] * cur.u[0];
 #pragma unroll
-        for (int q = 1; q < 4; ++q) l = __fma_rn(A[q], cur.u[q], l);
+        for (int q = 1; q < 4; ++q) l += A[q] * cur.u[q];
       }
       double lr[4];  // row r of L_ik
 #pragma unroll
@@ -413,10 +418,10 @@ __global__ void __launch_bounds__(32 * kFacWarps) k_ilu_factor_pair(
       // A_ij -= L_ik U_kj
       auto update = [&](int m, const double* w) {
         const int at = m < nm ? 16 * (int)mt[m0 + m] + hl : 0;
-        double x = m < nm ? bi[at] : 0.0;
+        double p = lr[0] * w[0];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) x = __fma_rn(-lr[q], w[q], x);
-        if (m < nm) bi[at] = x;
+        for (int q = 1; q < 4; ++q) p += lr[q] * w[q];
+        if (m < nm) bi[at] -= p;
       };
 #pragma unroll
       for (int m = 0; m < kAhead; ++m)

@@ -47,3 +47,8 @@ def _ilu_kernel(tmp_path):
 def test_ilu_two_rows_per_warp(tmp_path):
     _ilu_kernel(tmp_path)
     _run(tmp_path, "ilu.cpp")
+
+
+def test_ilu_two_rows_per_warp_rounds_as_the_definition(tmp_path):
+    _ilu_kernel(tmp_path)
+    _run(tmp_path, "ilu.cpp", "bits")

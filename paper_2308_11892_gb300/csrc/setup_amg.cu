@@ -2007,13 +2007,6 @@ __global__ void __launch_bounds__(1024) k_gauss_jordan(int n, double* __restrict
     for (int c = tx; c < n; c += 32) inv[(size_t)r * n + c] = M[(size_t)r * w + n + c];
 }
 
-// Gauss-Jordan on one cluster of kGjCtas CTAs, the augmented matrix [M | I]
-// held in their shared memory: CTA q owns columns [q w, q w + w) of the n x 2n
-// matrix (row-major slice).  Step k: the owner of column k finds the pivot in
-// its slice; after a cluster barrier every CTA reads the pivot row index and
-// the column-k factors through DSMEM; after a second barrier every CTA swaps,
-// scales and updates its own columns.  Same operations per element as
-// k_gauss_jordan, so the inverse is bit-identical to it.
 constexpr int kGjCtas = 16;
 constexpr int kGjThreads = 512;
 __device__ __forceinline__ void gj_cluster_sync() {
@@ -2050,12 +2043,16 @@ __device__ __forceinline__ void gj_push(V* local_ptr, unsigned rank, V v) {
 // every CTA has finished step k-2, so buffer k & 1 is free).  Each CTA then swaps,
 // scales and eliminates its own slice.
 //
+// The products and differences round one by one, like k_gauss_jordan's, whose inverse
+// this one equals bit for bit: a fused update would also decide otherwise which
+// matrices are singular (pure Neumann problems cancel down to the last pivot).
+//
 // The steps are a serial chain; each is bound by its CTA's FP64 rate (n w updates
-// at two per cycle) beside the barrier's latency, so an update is one fused
-// multiply-add, zeros are tested on the integer pipes, every column of every
-// slice is active, and no index is divided.  n = 208:
-// 1.40 -> 0.80 ms, n = 146: 0.68 -> 0.44 ms ([M | I] beside each other, an
-// FP64 compare, multiply and subtraction per element, before).
+// at two per cycle) beside the barrier's latency, so zeros are tested on the
+// integer pipes, every column of every slice is active, and no index is divided.
+// [M | I] beside each other and an FP64 compare per element took 1.40 ms at n = 208
+// and 0.68 at n = 146; in place with a fused update 0.80 and 0.44, which the separate
+// roundings lengthen by a fifth (64x64x32 grid's coarsest level 1.55 -> 1.87 ms).
 __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int w,
                                                                      const double* __restrict__ M,
                                                                      double* __restrict__ inv,
@@ -2132,7 +2129,7 @@ __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int 
       const double f = fcol[r];
       if (!d_eq0(f)) {
         const double a = cc == kc ? 0.0 : S[r * w + cc];
-        S[r * w + cc] = __fma_rn(-f, S[k * w + cc], a);
+        S[r * w + cc] = a - f * S[k * w + cc];
       }
       r += dr;
       cc += dc;
@@ -3100,7 +3097,7 @@ cptr_status setup_amg(cptr_ctx* c) {
       CTX_ALLOC(c, M, double, 2 * (size_t)nn * nn + 1, true);
       CTX_ALLOC(c, c->Cinv, double, (size_t)nn * nn + 1, true);
       KL(c, k_dense_fill<<<nblk(nn), kT, 0, c->stream>>>(nn, Lc->A.rp, Lc->A.ci, Lc->A.v, M));
-      // one cluster holding the whole augmented matrix when it fits, else one block
+      // one cluster holding the whole matrix when it fits (n <= 609), else one block
       bool clustered = false;
       {
         const int w = (nn + kGjCtas - 1) / kGjCtas;

@@ -83,3 +83,82 @@ def test_ilu_factors_have_the_definition_s_bits(P, oracle_mod, name):
     with P.Solver(n, rp, ci, v, precond=P.PREC_ILU).setup() as g:
         F = g.copy(0, P.COPY_ILU, np.float64, 16 * len(ci))
     np.testing.assert_array_equal(F.ravel(), np.asarray(o.ilu_factors()).ravel())
+
+
+def gauss_jordan(A):
+    """The definition of the coarsest inverse: [A | I], partial pivoting (largest |a|,
+    the first on ties), every product and difference rounded; None when singular."""
+    n = len(A)
+    a = np.concatenate([A, np.eye(n)], axis=1)
+    for k in range(n):
+        p = k + int(np.argmax(np.abs(a[k:, k])))
+        if not abs(a[p, k]) > 0.0:
+            return None
+        a[[k, p]] = a[[p, k]]
+        a[k] = a[k] / a[k, k]
+        f = a[:, k].copy()
+        f[k] = 0.0
+        a = a - f[:, None] * a[k][None, :]
+    return a[:, n:]
+
+
+def pressure_system(L):
+    """4x4 blocks with L in the first unknown and the identity in the others, so that
+    the first stage's scalar operator is L itself."""
+    n = len(L)
+    i, j = np.nonzero((L != 0) | np.eye(n, dtype=bool))
+    v = np.zeros((i.size, 4, 4))
+    v[:, 0, 0] = L[i, j]
+    v[i == j] += np.diag([0.0, 1.0, 1.0, 1.0])
+    rp = np.zeros(n + 1, np.int32)
+    np.cumsum(np.bincount(i, minlength=n), out=rp[1:])
+    return n, rp, j.astype(np.int32), v.reshape(-1, 16)
+
+
+def neumann(nx, ny, seed):
+    """Five-point operator without a boundary condition: its rows sum to zero."""
+    r = np.random.default_rng(seed)
+    n = nx * ny
+    L = np.zeros((n, n))
+    for i in range(n):
+        for j in ([i + 1] if (i + 1) % nx else []) + ([i + nx] if i + nx < n else []):
+            L[i, j] = L[j, i] = -r.uniform(0.5, 2.0)
+    for i in range(n):
+        for j in np.nonzero(L[i])[0]:
+            if j != i:
+                L[i, i] -= L[i, j]
+    return L
+
+
+def test_coarsest_operator_that_cancels(P):
+    answers = set()
+    for seed in range(200):
+        r = np.random.default_rng(seed)
+        L = neumann(int(r.integers(2, 8)), int(r.integers(2, 8)), seed)
+        want = P._lib.OK if gauss_jordan(L) is not None else P._lib.ERR_BREAKDOWN
+        answers.add(want)
+        assert _setup_status(P, *pressure_system(L), precond=P.PREC_FIRST, e1=-1) == want, seed
+    assert len(answers) == 2
+
+
+# one, two and 17 CTAs' worth of columns, slices with and without a remainder, the
+# largest matrix of the cluster (609) and the one-block kernel's smallest
+@pytest.mark.parametrize("n", [1, 15, 16, 17, 100, 209, 609, 610])
+def test_coarsest_inverse_has_the_definition_s_bits(P, n):
+    import torch
+    r = np.random.default_rng(n)
+    A = r.uniform(-1, 1, (n, n))
+    A[r.uniform(size=(n, n)) < 0.5] = 0.0
+    A[np.arange(n), np.arange(n)] = r.uniform(-1, 1, n)  # rows are exchanged
+    want = gauss_jordan(A)
+    cols = sorted({0, n // 3, n // 2, n - 1})
+    with P.Solver(*pressure_system(A), precond=P.PREC_FIRST, e1=-1, max_coarse=1024).setup() as g:
+        assert len(g.levels()) == 1
+        for c in cols:
+            b = torch.zeros(n, dtype=torch.float64, device="cuda")
+            b[c] = 1.0
+            x = torch.zeros_like(b)
+            torch.cuda.synchronize()
+            P.cptr_apply(g.h, P.APPLY_VCYCLE, b, x)
+            torch.cuda.synchronize()
+            np.testing.assert_array_equal(x.cpu().numpy(), want[:, c])

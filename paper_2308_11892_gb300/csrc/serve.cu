@@ -103,11 +103,10 @@ struct cptr_server {
   bool stop = false;
   std::string err;  // the last failed request's message
 
-  void note_failure(const Request& r, cptr_ctx* c, cptr_status st) {
+  void note_failure(const Request& r, const std::string& why, cptr_status st) {
     std::string m = "request " + std::to_string(r.id) + " (" + std::to_string(r.N) +
                      " cells): " + cptr_status_str(st);
-    const char* e = c ? cptr_last_error(c) : "";
-    if (e && *e) m += std::string(": ") + e;
+    if (!why.empty()) m += ": " + why;
     std::lock_guard<std::mutex> lk(mu);
     err = m;
   }
@@ -188,7 +187,7 @@ struct cptr_server {
     if (c) cptr_get_info(c, &r.info);
     r.info.status = st;
     r.st = st;
-    note_failure(r, c, st);
+    note_failure(r, c ? cptr_last_error(c) : "", st);
     cptr_destroy(c);
     return false;
   }
@@ -203,7 +202,7 @@ struct cptr_server {
     else if (c) cptr_get_info(c, &r.info);
     r.info.status = st;
     r.st = st;
-    if (st != CPTR_OK && st != CPTR_ERR_MAXIT) note_failure(r, c, st);
+    if (st != CPTR_OK && st != CPTR_ERR_MAXIT) note_failure(r, c ? cptr_last_error(c) : "", st);
     cptr_destroy(c);
     finish(r);
   }
@@ -233,6 +232,7 @@ struct cptr_server {
       // tol and maxit <= 0: each context's own (the request's)
       cptr_status st = cptr_solve_batch(cs.data(), n, rhs.data(), xs.data(), 0.0, 0, infos.data());
       const bool launched = st == CPTR_OK || st == CPTR_ERR_MAXIT || st == CPTR_ERR_BREAKDOWN;
+      const std::string why = cptr_last_error(cs[0]);  // (the loop destroys the contexts)
       for (int k = 0; k < n; ++k) {
         Request& r = *b[k];
         if (launched) {
@@ -242,7 +242,7 @@ struct cptr_server {
           cptr_get_info(r.ctx, &r.info);
           r.st = st;
           r.info.status = st;
-          note_failure(r, cs[0], st);
+          note_failure(r, why, st);
         }
         cptr_destroy(r.ctx);
         r.ctx = nullptr;

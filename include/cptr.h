@@ -181,8 +181,8 @@ cptr_status cptr_solve(cptr_ctx* c, const double* rhs, double* x, double tol, in
                        cptr_info* info);
 
 /* Solves n small systems at once on the device: one thread block, or a cluster of
- * up to eight, per system runs the whole flexible GMRES(restart) loop with the Eq. 3 preconditioner on the
- * device (block SpMV, restriction, V-cycle, correction, ILU(0) level by level,
+ * up to eight, per system runs the whole flexible GMRES(restart) loop with the
+ * Eq. 3 preconditioner on the device (block SpMV, restriction, V-cycle, correction, ILU(0) level by level,
  * CGS2, Givens rotations, restarts, true residual), with no host
  * synchronisation per iteration; the systems advance concurrently.  The same
  * algorithm and stopping rules as cptr_solve, with sums in a fixed order that
@@ -195,9 +195,11 @@ cptr_status cptr_solve(cptr_ctx* c, const double* rhs, double* x, double tol, in
  * guess, out: solution) are 4 N_k doubles, host or device.  tol <= 0 and
  * maxit <= 0 select each context's parameters.  infos (n entries) may be NULL.
  * Runs on the stream of ctxs[0] after every context's earlier work; returns
- * CPTR_OK when all converged, else the first failure (a breakdown before
- * CPTR_ERR_MAXIT); every x[k] is written.  Meant for systems of up to tens of
- * thousands of cells: one block or cluster per system. */
+ * CPTR_OK when all converged, else the first failure (CPTR_ERR_BREAKDOWN or
+ * CPTR_ERR_TIMEOUT before CPTR_ERR_MAXIT); every x[k] and infos[k] is written.
+ * CPTR_ERR_TIMEOUT: a system on a cluster waited longer for one of its rows than
+ * its limit (cptr_set_spin_limit); the other systems are solved as usual.  Meant
+ * for systems of up to tens of thousands of cells. */
 cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const double* const* rhs,
                              double* const* x, double tol, int maxit, cptr_info* infos);
 

@@ -1015,7 +1015,7 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
     if (infos) infos[k] = c->info;
     if (ho[k].status == CPTR_ERR_TIMEOUT)
       ctx_set_err(c0, "a bounded device-side wait gave up");
-    if (ho[k].status != CPTR_OK && (worst == CPTR_OK || ho[k].status != CPTR_ERR_MAXIT))
+    if (worst == CPTR_OK || (worst == CPTR_ERR_MAXIT && ho[k].status != CPTR_OK))
       worst = (cptr_status)ho[k].status;
   }
   return worst;

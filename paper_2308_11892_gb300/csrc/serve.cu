@@ -231,13 +231,17 @@ struct cptr_server {
       }
       // tol and maxit <= 0: each context's own (the request's)
       cptr_status st = cptr_solve_batch(cs.data(), n, rhs.data(), xs.data(), 0.0, 0, infos.data());
-      const bool launched = st == CPTR_OK || st == CPTR_ERR_MAXIT || st == CPTR_ERR_BREAKDOWN;
+      // these are systems' own statuses, after every system has its result; any other
+      // status is the batch's
+      const bool launched = st == CPTR_OK || st == CPTR_ERR_MAXIT ||
+                            st == CPTR_ERR_BREAKDOWN || st == CPTR_ERR_TIMEOUT;
       const std::string why = cptr_last_error(cs[0]);  // (the loop destroys the contexts)
       for (int k = 0; k < n; ++k) {
         Request& r = *b[k];
         if (launched) {
           r.info = infos[k];
           r.st = (cptr_status)infos[k].status;
+          if (r.st == CPTR_ERR_TIMEOUT) note_failure(r, why, r.st);
         } else {
           cptr_get_info(r.ctx, &r.info);
           r.st = st;

@@ -34,3 +34,9 @@ def test_failed_batch_keeps_its_message(tmp_path):
     """Every request of a batch that fails as a whole reports it; the message is read
     while the context that holds it exists."""
     _run(tmp_path, "fail")
+
+
+def test_timed_out_system_fails_alone(tmp_path):
+    """A system whose wait gave up, like one that broke down, leaves the other requests
+    of its batch their results."""
+    _run(tmp_path, "timeout")

@@ -19,6 +19,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -68,17 +69,26 @@ struct BOut {
   double rel_resid;
 };
 
-// A system runs on one cluster of 1, 2, 4 or 8 blocks (see cptr_solve_batch):
-// every loop over rows is dealt over the cluster's threads, and a phase ends at a
-// cluster barrier, which also makes the blocks' writes to global memory visible.
+// A system runs on one block (Solo) or on a cluster of 2, 4 or 8 (Team; see
+// cptr_solve_batch): every loop over rows is dealt over its threads, and a phase ends at
+// its barrier, which also makes the blocks' writes to global memory visible.
 // A row's sum never depends on the dealing, and the dots and norms are cut into
 // kParts slices of the rows whatever the number of blocks, so the result is the
 // same on any cluster size.
 //
 // One block is bound by its SM's FP64 rate (outer SpMV, CGS2) and by memory
-// latency (V-cycle rows, ILU(0) levels); the cluster divides the first by its
-// size, and the levels read what does not depend on the level before ahead of
-// the barrier.
+// latency (V-cycle rows, ILU(0) levels); the cluster divides the first by its size.
+// The kernel is compiled for one block apart, in line throughout and with constant
+// strides: the clusters' code on one block took 30.5 instead of 21.7 ms for 152 grids of
+// 8,000 cells (mixed; 39.0 and 28.2 FP64), 6.6 instead of 5.0 for 48 of 1,859, 4.9
+// instead of 3.7 for one cloud of 507.  For a cluster every phase is a call: in line, the
+// polling loop of the ILU(0) solves loses 2-8% to the code around it (24 grids of 30k
+// cells on four blocks 29.2 instead of 27.5 ms).
+struct Solo {
+  static constexpr int rank = 0, size = 1, threads = kBT;
+  int tid = (int)threadIdx.x;
+  __device__ __forceinline__ void sync() const { __syncthreads(); }
+};
 struct Team {
   int rank, size;  // block of the cluster, blocks in it
   int tid, threads;
@@ -92,17 +102,25 @@ struct Team {
     threads = size * kBT;
   }
   __device__ __forceinline__ void sync() const {
-    if (size == 1) {
-      __syncthreads();
-    } else {
-      __syncwarp();
-      asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
-                   "barrier.cluster.wait.acquire.aligned;" ::: "memory");
-    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
+                 "barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+};
+// Phase<f>::run(t, ...): f in line on one block, a call on a cluster.
+template <auto F>
+struct Phase;
+template <class TM, class... A, void (*F)(const TM&, A...)>
+struct Phase<F> {
+  static __device__ __noinline__ void call(const TM& t, A... a) { F(t, a...); }
+  static __device__ __forceinline__ void run(const TM& t, A... a) {
+    if constexpr (std::is_same_v<TM, Solo>) F(t, a...);
+    else call(t, a...);
   }
 };
 // A double of another block's shared memory.
-__device__ __forceinline__ double team_read(const double* own, int rank) {
+__device__ __forceinline__ double team_read(const Solo&, const double* own, int) { return *own; }
+__device__ __forceinline__ double team_read(const Team&, const double* own, int rank) {
   unsigned a = (unsigned)__cvta_generic_to_shared(own), r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
   double v;
@@ -119,7 +137,10 @@ struct Partials {
 };
 
 // out[l] = V_l . w for l < nc (V_l = V + l n), the same in every block: a warp sums
-// G columns over one slice, the slices are combined by a shuffle tree.
+// G columns over one slice, the slices are combined by a shuffle tree.  The slices are
+// short (kParts of them whatever the blocks), so the columns share the tree of warp_sum:
+// its first two steps halve the columns a lane holds, with the same pairs of lanes added
+// for every column, in 6 additions for four columns instead of 20.
 template <int G>
 __device__ __forceinline__ void part_dot(const double* V, size_t n, const double* w, int lo,
                                          int hi, double* out) {
@@ -133,14 +154,24 @@ __device__ __forceinline__ void part_dot(const double* V, size_t n, const double
 #pragma unroll
     for (int u = 0; u < G; ++u) acc[u] += V[(size_t)u * n + i] * wi;
   }
+  // lanes with the bit of step o clear keep the even columns
+  auto halve = [&](double a, double b, int o) {
+    const bool high = lane & o;
+    return (high ? b : a) + __shfl_xor_sync(0xffffffffu, high ? a : b, o);
+  };
+  double s;
+  if (G == 1) s = acc[0] + __shfl_xor_sync(0xffffffffu, acc[0], 16);
+  else s = halve(acc[0], acc[G > 1 ? 1 : 0], 16);
+  if (G <= 2) s += __shfl_xor_sync(0xffffffffu, s, 8);
+  else s = halve(s, halve(acc[G > 2 ? 2 : 0], G > 3 ? acc[G > 3 ? 3 : 0] : 0.0, 16), 8);
 #pragma unroll
-  for (int u = 0; u < G; ++u) {
-    const double s = warp_sum(acc[u]);
-    if (lane == 0) out[u] = s;
-  }
+  for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  const int u = (lane >> 4 & 1) + (G > 2 ? 2 * (lane >> 3 & 1) : 0);
+  if ((lane & 7) == 0 && u < G && (G > 2 || (lane & 8) == 0)) out[u] = s;
 }
-__device__ __noinline__ void team_dots(const Team& t, Partials& P, const double* V, const double* w, int n,
-                          int nc, double* out) {
+template <class TM>
+__device__ __forceinline__ void team_dots(const TM& t, Partials& P, const double* V,
+                                          const double* w, int n, int nc, double* out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = kBT / 32;
   const int mine = kParts / t.size;
   const int per = ((n + kParts - 1) / kParts + 31) & ~31;
@@ -160,7 +191,7 @@ __device__ __noinline__ void team_dots(const Team& t, Partials& P, const double*
   }
   t.sync();
   for (int l = warp; l < nc; l += nw) {
-    const double s = warp_sum(team_read(part + (lane % mine) * (kBMaxM + 1) + l, lane / mine));
+    const double s = warp_sum(team_read(t, part + (lane % mine) * (kBMaxM + 1) + l, lane / mine));
     if (lane == 0) out[l] = s;
   }
   __syncthreads();
@@ -170,8 +201,9 @@ __device__ __noinline__ void team_dots(const Team& t, Partials& P, const double*
 
 // w -= V h over the first nc columns, four elements per thread at a time (their
 // loads overlap; each element takes its columns in order).
-__device__ __noinline__ void team_update(const Team& t, const double* V, double* w, int n, int nc,
-                                         const double* h) {
+template <class TM>
+__device__ __forceinline__ void team_update(const TM& t, const double* V, double* w, int n, int nc,
+                                            const double* h) {
   for (int i0 = t.tid; i0 < n; i0 += 4 * t.threads) {
     double wi[4];
 #pragma unroll
@@ -211,8 +243,9 @@ __device__ __forceinline__ void ld4x(const float* p, double* o) {  // (off the F
 }
 
 // y = A x (4x4 blocks, FP64 accumulation in block order), y = b - A x when b
-template <class TX>
-__device__ __noinline__ void bspmv(const Team& t, const BSys& S, const TX* x, const double* b, double* y) {
+template <class TM, class TX>
+__device__ __forceinline__ void bspmv(const TM& t, const BSys& S, const TX* x, const double* b,
+                                      double* y) {
   const int n4 = 4 * S.N;
   const int32_t* __restrict__ rp = S.rp;
   const int32_t* __restrict__ ci = S.ci;
@@ -252,8 +285,8 @@ __device__ __noinline__ void bspmv(const Team& t, const BSys& S, const TX* x, co
 // (a thread per row; four entries are loaded before their products are added.  Eight
 // at a time, predicated, took 62 million clocks against 49 in the V-cycles of a
 // 24.6k-cell cloud on one block; the last one to three are read together.)
-template <class T, class F>
-__device__ __forceinline__ void rows(const Team& t, int n, const int32_t* __restrict__ rp,
+template <class TM, class T, class F>
+__device__ __forceinline__ void rows(const TM& t, int n, const int32_t* __restrict__ rp,
                                      const int32_t* __restrict__ ci, const T* __restrict__ val,
                                      const T* x, F f) {
   for (int i = t.tid; i < n; i += t.threads) {
@@ -293,35 +326,35 @@ __device__ __forceinline__ void rows(const Team& t, int n, const int32_t* __rest
 }
 
 // r = b - A x on one AMG level (scalar CSR, apply precision)
-template <class T>
-__device__ __noinline__ void lresid(const Team& t, const BLevel& L, const T* b, const T* x, T* r) {
-  rows<T>(t, L.n, L.Arp, L.Aci, (const T*)L.Av, x, [=](int i, T s) { r[i] = b[i] - s; });
+template <class TM, class T>
+__device__ __forceinline__ void lresid(const TM& t, const BLevel& L, const T* b, const T* x, T* r) {
+  rows(t, L.n, L.Arp, L.Aci, (const T*)L.Av, x, [=](int i, T s) { r[i] = b[i] - s; });
 }
 
 // xout = xin + D_l1^-1 (b - A xin): one l1-Jacobi sweep
-template <class T>
-__device__ __noinline__ void lsweep(const Team& t, const BLevel& L, const T* b, const T* xin, T* xout) {
+template <class TM, class T>
+__device__ __forceinline__ void lsweep(const TM& t, const BLevel& L, const T* b, const T* xin, T* xout) {
   const T* dv = (const T*)L.dinv;
-  rows<T>(t, L.n, L.Arp, L.Aci, (const T*)L.Av, xin,
+  rows(t, L.n, L.Arp, L.Aci, (const T*)L.Av, xin,
           [=](int i, T s) { xout[i] = xin[i] + dv[i] * (b[i] - s); });
 }
 
 // b_{l+1} = R r and x += P xc
-template <class T>
-__device__ __noinline__ void lrestrict(const Team& t, const BLevel& L, const T* r, T* bn) {
+template <class TM, class T>
+__device__ __forceinline__ void lrestrict(const TM& t, const BLevel& L, const T* r, T* bn) {
   const int32_t *rp = L.Rrp, *ci = L.Rci;
   const T* rv = (const T*)L.Rv;
-  rows<T>(t, L.nc, rp, ci, rv, r, [=](int i, T s) { bn[i] = s; });
+  rows(t, L.nc, rp, ci, rv, r, [=](int i, T s) { bn[i] = s; });
 }
-template <class T>
-__device__ __noinline__ void lprolong(const Team& t, const BLevel& L, const T* xc, T* x) {
-  rows<T>(t, L.n, L.Prp, L.Pci, (const T*)L.Pv, xc, [=](int i, T s) { x[i] += s; });
+template <class TM, class T>
+__device__ __forceinline__ void lprolong(const TM& t, const BLevel& L, const T* xc, T* x) {
+  rows(t, L.n, L.Prp, L.Pci, (const T*)L.Pv, xc, [=](int i, T s) { x[i] += s; });
 }
 
 // One V(nu_pre, nu_post) cycle with l1-Jacobi from a zero guess on the
 // system's hierarchy: b0 (level 0 right-hand side) -> zc.
-template <class T>
-__device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) {
+template <class TM, class T>
+__device__ __forceinline__ void bvcycle(const TM& t, const BSys& S, const T* b0) {
   const int last = S.nlev - 1;
   for (int l = 0; l < last; ++l) {
     const BLevel& L = S.lev[l];
@@ -339,16 +372,16 @@ __device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) 
       for (int k = 1; k < S.nu_pre; ++k) {
         t.sync();
         T* d2 = ((S.nu_pre - 1 - k) % 2 == 0) ? x : tt;
-        lsweep<T>(t, L, b, src, d2);
+        Phase<lsweep<TM, T>>::run(t, L, b, src, d2);
         src = d2;
       }
     }
     t.sync();
-    lresid<T>(t, L, b, x, (T*)L.r);
+    Phase<lresid<TM, T>>::run(t, L, b, x, (T*)L.r);
     t.sync();
     // b_{l+1} = R r
     T* bn = (T*)S.lev[l + 1].b;
-    lrestrict<T>(t, L, (const T*)L.r, bn);
+    Phase<lrestrict<TM, T>>::run(t, L, (const T*)L.r, bn);
     t.sync();
   }
   {
@@ -375,7 +408,7 @@ __device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) 
     T* x = (T*)L.x;
     T* tt = (T*)L.t;
     T* out = l == 0 ? (T*)S.zc : (T*)L.x2;
-    lprolong<T>(t, L, xc, x);
+    Phase<lprolong<TM, T>>::run(t, L, xc, x);
     t.sync();
     if (S.nu_post == 0) {
       for (int i = t.tid; i < L.n; i += t.threads) out[i] = x[i];
@@ -383,7 +416,7 @@ __device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) 
       const T* src = x;
       for (int k = 0; k < S.nu_post; ++k) {
         T* dst = (k == S.nu_post - 1) ? out : (src == x ? tt : x);
-        lsweep<T>(t, L, b, src, dst);
+        Phase<lsweep<TM, T>>::run(t, L, b, src, dst);
         if (k + 1 < S.nu_post) t.sync();
         src = dst;
       }
@@ -396,140 +429,67 @@ __device__ __noinline__ void bvcycle(const Team& t, const BSys& S, const T* b0) 
 // rounding sequence.  A level is a few dozen rows, so a solve is the latency of its
 // levels, one after the other.
 //
-// One block (tri_solve) separates the levels by its barrier, and everything but the
-// solutions of earlier levels is on its way before a row is worked on: a row's
-// number and block range three levels ahead, its blocks to L2 two ahead and to
-// registers one ahead, behind the level's own gather, which they would delay in
-// front of it.  On a cluster a barrier that publishes global memory costs about
+// One block (tri_solve) separates the levels by its barrier.  (Reading the rows of the
+// coming levels ahead of the barrier made the solves of clouds up to a third shorter,
+// those of grids up to twice as long, and the other phases longer with its registers:
+// with everything else alike 27.7 instead of 21.9 ms for 152 grids of 8,000 cells, 22.0
+// instead of 23.0 for 152 clouds of 3,750.)  On a cluster a barrier that publishes global memory costs about
 // 5 us, so there (tri_solve_poll) the rows are dealt over the cluster's quads in
 // schedule order and wait for their dependencies' values instead (a sentinel until
-// they are written, read a bounded number of times); a quad has a row every few
-// levels and reads it ahead while it waits.  The quads take their rows in order and
-// the blocks of a cluster run together, so each wait ends: a 32k-point cloud (405
+// they are written, read a bounded number of times).  The quads take their rows in order
+// and the blocks of a cluster run together, so each wait ends: a 32k-point cloud (405
 // levels) on eight blocks, 7 iterations, 41.5 ms with a barrier per level, 25 ms so.
-struct RowMeta {
-  int p, i, kb, ke;
-};
-__device__ __forceinline__ RowMeta row_meta(int p, int pe, const int32_t* __restrict__ ord,
-                                            const int32_t* __restrict__ rp) {
-  RowMeta m{p, -1, 0, 0};
-  if (p < pe) {
-    m.i = ord[p];
-    m.kb = rp[p];
-    m.ke = rp[p + 1];
-  }
-  return m;
-}
-template <class T>
-struct TriRow {
-  static constexpr int kPre = sizeof(T) == 4 ? 6 : 3;  // dependencies read ahead (registers)
-  int p, i, kb, ke;
-  T acc;
-  int j[kPre];
-  T f[kPre][4];
-};
-template <class T>
-__device__ __forceinline__ void row_data(TriRow<T>& R, const RowMeta& m,
-                                         const int32_t* __restrict__ ci,
-                                         const T* __restrict__ F, const T* rhs, int r) {
-  R.p = m.p;
-  R.i = m.i;
-  R.kb = R.ke = 0;
-  R.acc = 0;
-  if (m.i < 0) return;
-  R.kb = m.kb;
-  R.ke = m.ke;
-  R.acc = rhs[4 * (size_t)m.i + r];
-#pragma unroll
-  for (int u = 0; u < TriRow<T>::kPre; ++u)
-    if (m.kb + u < m.ke) {
-      R.j[u] = ci[m.kb + u];
-      ld4(F + 16 * (size_t)(m.kb + u) + 4 * r, R.f[u]);
-    }
-}
-// the row's right-hand side minus its blocks times the solutions, in block order
-template <class T>
-__device__ __forceinline__ T row_finish(const TriRow<T>& R, const int32_t* __restrict__ ci,
-                                        const T* __restrict__ F, const T* y, int r) {
-  T acc = R.acc;
-  T x[TriRow<T>::kPre][4];
-#pragma unroll
-  for (int u = 0; u < TriRow<T>::kPre; ++u)
-    if (R.kb + u < R.ke) ld4x(y + 4 * (size_t)R.j[u], x[u]);
-#pragma unroll
-  for (int u = 0; u < TriRow<T>::kPre; ++u)
-    if (R.kb + u < R.ke) acc = sub_rn(acc, dot4(R.f[u], x[u]));
-  for (int k = R.kb + TriRow<T>::kPre; k < R.ke; k += 3) {
-    T f[3][4], xx[3][4];
-#pragma unroll
-    for (int u = 0; u < 3; ++u)
-      if (k + u < R.ke) {
-        ld4(F + 16 * (size_t)(k + u) + 4 * r, f[u]);
-        ld4x(y + 4 * (size_t)ci[k + u], xx[u]);
-      }
-#pragma unroll
-    for (int u = 0; u < 3; ++u)
-      if (k + u < R.ke) acc = sub_rn(acc, dot4(f[u], xx[u]));
-  }
-  return acc;
-}
+//
 // Forward: y = L^-1 rhs.  Backward (UPPER): y = U^-1 rhs and z = P zc + y.
 template <class T, bool UPPER>
-__device__ __noinline__ void tri_solve(const Team& t, const BSys& S, const T* rhs, T* y, T* z) {
-  const int32_t* __restrict__ off = UPPER ? S.offb : S.offf;
-  const int32_t* __restrict__ ord = UPPER ? S.ordb : S.ordf;
-  const int32_t* __restrict__ rp = UPPER ? S.Urp : S.Lrp;
-  const int32_t* __restrict__ ci = UPPER ? S.Uci : S.Lci;
-  const T* __restrict__ F = (const T*)(UPPER ? S.Uv : S.Lv);
+__device__ __forceinline__ void tri_solve(const Solo&, const BSys& S, const T* rhs, T* y, T* z) {
+  const int32_t* off = UPPER ? S.offb : S.offf;
+  const int32_t* ord = UPPER ? S.ordb : S.ordf;
+  const int32_t* rp = UPPER ? S.Urp : S.Lrp;
+  const int32_t* ci = UPPER ? S.Uci : S.Lci;
+  const T* F = (const T*)(UPPER ? S.Uv : S.Lv);
   const int nl = UPPER ? S.nlb : S.nlf;
-  const int r = threadIdx.x & 3, quad = t.tid >> 2, nquad = t.threads >> 2;
+  const int r = threadIdx.x & 3, quad = threadIdx.x >> 2, nquad = kBT >> 2;
   const unsigned qmask = 0xFu << ((threadIdx.x & 31) & ~3);
   const int q0 = (threadIdx.x & 31) & ~3;
-  // level lv: positions [o0, o1), the next ones [o1, o2), [o2, o3), [o3, o4)
-  int o0 = off[0], o1 = off[1], o2 = off[min(2, nl)], o3 = off[min(3, nl)];
-  TriRow<T> R;
-  row_data<T>(R, row_meta(o0 + quad, o1, ord, rp), ci, F, rhs, r);
-  RowMeta m1 = row_meta(o1 + quad, o2, ord, rp), m2 = row_meta(o2 + quad, o3, ord, rp);
   for (int lv = 0; lv < nl; ++lv) {
-    for (int p = o0 + quad;;) {
+    const int pe = off[lv + 1];
+    for (int p = off[lv] + quad; p < pe; p += nquad) {
+      const int i = ord[p];
+      if (i < 0) continue;
       T d[4] = {0, 0, 0, 0}, y1 = 0;
-      if (UPPER && R.i >= 0) {
-        // inv(U_ii) and the first-stage part, beside the gather
-        ld4((const T*)S.Dinv + 16 * (size_t)R.p + 4 * r, d);
+      if (UPPER) {
+        // inv(U_ii) and the first-stage part before the row's sums
+        const T* dp = (const T*)S.Dinv + 16 * (size_t)p + 4 * r;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) d[q] = dp[q];
         if (S.first) {
           const T* zc = (const T*)S.zc;
-          if (r == S.e0) y1 = zc[S.ne * (size_t)R.i];
-          else if (S.ne == 2 && r == S.e1) y1 = zc[2 * (size_t)R.i + 1];
+          if (r == S.e0) y1 = zc[S.ne * (size_t)i];
+          else if (S.ne == 2 && r == S.e1) y1 = zc[2 * (size_t)i + 1];
         }
       }
-      T acc = R.i >= 0 ? row_finish(R, ci, F, y, r) : T(0);
+      T acc = rhs[4 * (size_t)i + r];
+      for (int k = rp[p]; k < rp[p + 1]; ++k) {
+        T f[4], yj[4];
+        const T* fp = F + 16 * (size_t)k + 4 * r;
+        const T* yp = y + 4 * (size_t)ci[k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          f[q] = fp[q];
+          yj[q] = yp[q];
+        }
+        acc = sub_rn(acc, dot4(f, yj));
+      }
       if (UPPER) {
         T s4[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) s4[q] = __shfl_sync(qmask, acc, q0 + q);
         acc = dot4(d, s4);
+        z[4 * (size_t)i + r] = y1 + acc;
       }
-      if (R.i >= 0) {
-        y[4 * (size_t)R.i + r] = acc;
-        if (UPPER) z[4 * (size_t)R.i + r] = y1 + acc;
-      }
-      p += nquad;
-      if (p >= o1) break;
-      row_data<T>(R, row_meta(p, o1, ord, rp), ci, F, rhs, r);
+      y[4 * (size_t)i + r] = acc;
     }
-    // in flight behind the barrier: the next level's row, the row numbers three
-    // levels ahead, and the blocks two levels ahead on their way to L2
-    row_data<T>(R, m1, ci, F, rhs, r);
-    const int o4 = off[min(lv + 4, nl)];
-    for (int k = m2.kb + r; k < m2.ke; k += 4) {
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(F + 16 * (size_t)k));
-      if (sizeof(T) == 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(F + 16 * (size_t)k + 8));
-    }
-    if (UPPER && m2.i >= 0 && r == 0)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"((const T*)S.Dinv + 16 * (size_t)m2.p));
-    m1 = m2;
-    m2 = row_meta(o3 + quad, o4, ord, rp);
-    o0 = o1; o1 = o2; o2 = o3; o3 = o4;
     __syncthreads();
   }
 }
@@ -606,8 +566,8 @@ __device__ __noinline__ void tri_solve_poll(const Team& t, const BSys& S, const 
 }
 
 // z = M^-1 v (Eq. 3) for the FP64 vector v; z in the apply precision.
-template <class T>
-__device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double* v, T* z) {
+template <class TM, class T>
+__device__ __forceinline__ void bprecond(const TM& t, const BSys& S, const double* v, T* z) {
   const int N = S.N;
   T* rhat = (T*)S.rhat;
   T* zc = (T*)S.zc;
@@ -629,7 +589,7 @@ __device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double
       }
     }
     t.sync();
-    bvcycle<T>(t, S, rhat);
+    Phase<bvcycle<TM, T>>::run(t, S, rhat);
     // correction: r2 = v - A P zc (elliptic columns of A only)
     const T* __restrict__ ae = (const T*)S.AE;
     const int32_t* __restrict__ rp = S.rp;
@@ -671,15 +631,15 @@ __device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double
   } else {
     for (int g = t.tid; g < 4 * N; g += t.threads) r2[g] = (T)v[g];
   }
-  if (t.size > 1)
-    for (int g = t.tid; g < 4 * N; g += t.threads) u[g] = sentinel_of(T(0));
-  t.sync();
-  if (t.size > 1) {
-    tri_solve_poll<T, false>(t, S, r2, u, y2, nullptr);
-    tri_solve_poll<T, true>(t, S, u, y2, nullptr, z);
-  } else {
+  if constexpr (std::is_same_v<TM, Solo>) {
+    t.sync();
     tri_solve<T, false>(t, S, r2, u, nullptr);
     tri_solve<T, true>(t, S, u, y2, z);
+  } else {
+    for (int g = t.tid; g < 4 * N; g += t.threads) u[g] = sentinel_of(T(0));
+    t.sync();
+    tri_solve_poll<T, false>(t, S, r2, u, y2, nullptr);
+    tri_solve_poll<T, true>(t, S, u, y2, nullptr, z);
   }
 }
 
@@ -690,10 +650,10 @@ __device__ __noinline__ void bprecond(const Team& t, const BSys& S, const double
 // maxit or on an exact breakdown, and the true residual decides whether to
 // start another.  Every block keeps the Hessenberg matrix and takes the same
 // decisions from the same sums.
-template <class T>
+template <class T, class TM>
 __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict__ sys,
                                                       BOut* __restrict__ out) {
-  const Team t;
+  const TM t;
   const int id = blockIdx.x / t.size;
   // the system's descriptor in shared memory: its pointers are then read
   // without a global load, and stores to global memory cannot alias them
@@ -714,7 +674,7 @@ __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict_
   const int tid = threadIdx.x;
   T* Z = (T*)S.Z;
   // ||b||
-  team_dots(t, P, S.b, S.b, n4, 1, snrm);
+  Phase<team_dots<TM>>::run(t, P, S.b, S.b, n4, 1, snrm);
   const double bnorm = sqrt(snrm[0]);
   const double tol_abs = S.tol * bnorm;
   int iters = 0, status = CPTR_OK;
@@ -724,9 +684,9 @@ __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict_
   } else {
     for (;;) {
       // r = b - A x into V_0, beta = ||r||
-      bspmv<double>(t, S, S.x, S.b, S.V);
+      Phase<bspmv<TM, double>>::run(t, S, S.x, S.b, S.V);
       t.sync();
-      team_dots(t, P, S.V, S.V, n4, 1, snrm);
+      Phase<team_dots<TM>>::run(t, P, S.V, S.V, n4, 1, snrm);
       beta = sqrt(snrm[0]);
       if (!isfinite(beta)) { status = CPTR_ERR_BREAKDOWN; break; }
       if (beta <= tol_abs) break;
@@ -741,21 +701,21 @@ __global__ void __launch_bounds__(kBT, 1) k_batch_fgmres(const BSys* __restrict_
       for (int j = 0; j < m; ++j) {
         const double* vj = S.V + (size_t)j * n4;
         T* zj = Z + (size_t)j * n4;
-        bprecond<T>(t, S, vj, zj);
+        Phase<bprecond<TM, T>>::run(t, S, vj, zj);
         if (t.size > 1 && ld_volatile_i32(S.fail)) {  // (set before the last barrier)
           status = CPTR_ERR_TIMEOUT;
           break;
         }
-        bspmv<T>(t, S, zj, nullptr, S.w);
+        Phase<bspmv<TM, T>>::run(t, S, zj, nullptr, S.w);
         t.sync();
         // CGS2: h1 = V^T w; w -= V h1; h2 = V^T w; w -= V h2
         for (int pass = 0; pass < 2; ++pass) {
           double* hh = pass == 0 ? sh1 : sh2;
-          team_dots(t, P, S.V, S.w, n4, j + 1, hh);
-          team_update(t, S.V, S.w, n4, j + 1, hh);
+          Phase<team_dots<TM>>::run(t, P, S.V, S.w, n4, j + 1, hh);
+          Phase<team_update<TM>>::run(t, S.V, S.w, n4, j + 1, hh);
           t.sync();
         }
-        team_dots(t, P, S.w, S.w, n4, 1, snrm);
+        Phase<team_dots<TM>>::run(t, P, S.w, S.w, n4, 1, snrm);
         const double hn = sqrt(snrm[0]);
         if (tid == 0) {
           double* col = sH + (size_t)j * (m + 1);
@@ -976,12 +936,12 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = size > 1 ? 1 : 0;
     const BSys* sy = dsys + k0;
+    auto kern = c0->mixed ? (size > 1 ? k_batch_fgmres<float, Team> : k_batch_fgmres<float, Solo>)
+                          : (size > 1 ? k_batch_fgmres<double, Team> : k_batch_fgmres<double, Solo>);
     e = cudaStreamWaitEvent(lead->stream2, c0->ev_fork, 0);
-    if (e == cudaSuccess)
-      e = c0->mixed ? cudaLaunchKernelEx(&cfg, k_batch_fgmres<float>, sy, dout + k0)
-                    : cudaLaunchKernelEx(&cfg, k_batch_fgmres<double>, sy, dout + k0);
+    if (e == cudaSuccess) e = cudaLaunchKernelEx(&cfg, kern, sy, dout + k0);
     ++c0->nlaunch;
     // (also after a failed launch: what runs on the other streams is waited for)
     if (cudaEventRecord(lead->ev_join, lead->stream2) != cudaSuccess ||

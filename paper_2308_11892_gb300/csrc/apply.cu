@@ -687,17 +687,29 @@ void launch_ilu_levels(cptr_ctx* c, const T* zc, void* zbase, const int* jptr, s
   //     1.65 / 2.64 (1.94 / 3.88);
   //   FP64, 150x110x57 grid (2986 rows): 0.53 / 0.63 against 0.61 / 0.70
   //     (0.67 / 1.07); 200x200x100 grid: 1.66 / 1.93 against 1.14 / 1.32.
+  //
+  // Where no row has more than five blocks (lines and plane grids: one and two
+  // dependencies), a batch of two, or of one on a line, with four lanes: the longer
+  // batches' unused products still take their slots of the FP64 pipe, and on these
+  // shapes nothing hides them.  One application, against 16 lanes in FP64 and a batch
+  // of three in FP32: line of 500 cells 0.60 / 0.96 and 0.44 / 0.49 ms (one read after
+  // the other: 0.64 and 0.50), 20x20 0.086 / 0.104 and 0.061 / 0.063, 300x300
+  // 1.58 / 1.70 and 1.01 / 1.06, 700x700 3.81 / 4.04 and 2.46 / 2.63.
   const bool f32 = sizeof(T) == 4;
   const long long rows = c->nlev_f > 0 ? c->N / c->nlev_f : c->N;
   const bool narrow = rows <= 32ll * c->nsm;
   const bool long_rows = 2 * c->nnzL > 7ll * c->N;  // over 3.5 dependencies on average
   const int forced = c->lvl_grid_forced;
-  if (narrow && (!f32 || long_rows))
+  const int grid4 = forced ? forced : (f32 ? 3 : 2) * c->nsm;
+  if (narrow && c->max_row <= 3 && c->nnzL <= c->N)
+    launch_levels_as<T, 4, 1>(c, grid4, zc, zbase, jptr, stride, active, which);
+  else if (narrow && c->max_row <= 5 && c->nnzL <= 2ll * c->N)
+    launch_levels_as<T, 4, 2>(c, grid4, zc, zbase, jptr, stride, active, which);
+  else if (narrow && (!f32 || long_rows))
     launch_levels_as<T, 16, sizeof(T) == 4 ? 2 : 1>(c, forced ? forced : (f32 ? 2 : 3) * c->nsm,
                                                     zc, zbase, jptr, stride, active, which);
   else
-    launch_levels_as<T, 4, 3>(c, forced ? forced : (f32 ? 3 : 2) * c->nsm, zc, zbase, jptr,
-                              stride, active, which);
+    launch_levels_as<T, 4, 3>(c, grid4, zc, zbase, jptr, stride, active, which);
 }
 
 // which: 0 = forward and backward, 1 = forward only, 2 = backward only

@@ -214,6 +214,7 @@ struct cptr_ctx {
   int32_t* lvl_f = nullptr;
   int32_t* lvl_b = nullptr;
   int nlev_f = 0, nlev_b = 0;
+  int max_row = 0;                     // blocks of A's longest row
   int npos_f = 0, npos_b = 0;          // padded schedule lengths
   int32_t* ord_f = nullptr;            // schedule position -> row (-1 = padding)
   int32_t* ord_b = nullptr;

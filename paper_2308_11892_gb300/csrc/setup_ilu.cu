@@ -618,6 +618,7 @@ cptr_status setup_ilu_factor(cptr_ctx* c) {
   int hm = 0;
   CTX_CUDA(c, cudaMemcpyAsync(&hm, mrow, sizeof(int), cudaMemcpyDeviceToHost, cs(c)));
   CTX_CUDA(c, cudaStreamSynchronize(cs(c)));
+  c->max_row = hm;
   if (hm <= kRowMax && !c->force_fallback) {
     const FacRow lay = fac_row(hm);
     KL(c, k_ilu_factor_pair<<<c->nsm * 8, 32 * kFacWarps, (size_t)lay.bytes * 2 * kFacWarps,

@@ -1,15 +1,14 @@
-// Batched solves of many small systems in one launch.
+// Batched solves of many small systems at once.
 //
 // A small system (thousands of cells) leaves most of the GPU idle in the
 // per-system path, whose Krylov loop launches a few dozen kernels per
 // iteration and reads a host flag at every restart.  Here one thread block, or a
 // cluster of up to eight, runs the whole flexible GMRES(m) loop of one system on
-// the device, with the
-// Eq. 3 preconditioner (Quasi-IMPES restriction, the system-AMG V-cycle, the
-// correction, the ILU(0) solves level by level, the combination), the outer
-// block SpMV, CGS2 with Givens rotations, the back substitution, restarts and
-// the true residual, separated by block or cluster barriers only; a grid of them
-// advances every system of the batch at once.  Each system reads its own
+// the device, with the Eq. 3 preconditioner (Quasi-IMPES restriction, the
+// system-AMG V-cycle, the correction, the ILU(0) solves, the combination), the
+// outer block SpMV, CGS2 with Givens rotations, the back substitution, restarts
+// and the true residual, with no host in between; a grid of them advances every
+// system of the batch at once.  Each system reads its own
 // context's hierarchy, factors and work vectors (built by cptr_setup), and
 // every sum has a fixed order that does not depend on the batch: a system's
 // result is the same alone and in any batch.
@@ -878,18 +877,19 @@ extern "C" cptr_status cptr_solve_batch(cptr_ctx* const* ctxs, int n, const doub
     CTX_CUDA(c0, cudaMemcpyAsync(ctxs[k]->bd, rhs[k], nb, cudaMemcpyDefault, s));
     CTX_CUDA(c0, cudaMemcpyAsync(ctxs[k]->xd, x[k], nb, cudaMemcpyDefault, s));
   }
-  // Blocks per system, in proportion to its cells, so that the batch's largest
-  // system does not run alone on one SM when the others are done: 1, 2, 4 or 8, a
-  // block for every 0.6 of an SM's share of the batch's cells (with fewer the last
-  // systems leave SMs idle, with more the barriers cost more than they divide: 48
-  // systems of 2k-30k cells took 42, 39, 41 and 129 ms with 0.5, 0.7, 1 share and
-  // one block each, 120 systems of 2k-20k 58, 55, 64 and 118 ms, 200 of 2k-30k 115,
-  // 137, 160 and 202 ms; the 48 take 31 ms with 0.6) and at least
-  // kBlockCells cells.  From kMostCells on a block is divided whatever the batch: it
-  // loses more to its L1 than the barriers cost (304 systems of 2k-28k cells: 178 ms
-  // without this limit, 132 with 5632, 127 with 4096; 160 systems 90, 90, 78).
-  // Systems are laid out by that number and each group is one launch, side by side
-  // on its first system's second stream.
+  // Blocks per system: the largest of 1, 2, 4 and 8 whose blocks hold at least a share of
+  // cells each, so that the batch's largest system does not run alone on one SM when the
+  // others are done; a block then holds fewer than two shares, but for systems of more
+  // than sixteen.  A share is 0.6 of the cells per SM of the batch: with larger ones the
+  // last systems leave SMs idle, with smaller ones the barriers cost more than they
+  // divide (48 systems of 2k-30k cells take 27.9, 28.1, 27.7 and 36.5 ms with 0.5, 0.6, 0.7
+  // and 1, 93.5 with one block each; 120 of 2k-20k 35.3, 35.7, 33.6, 33.7 and 57.9).  It
+  // is at least kBlockCells, and at most kMostCells, whatever the batch: a block of many
+  // cells loses more to its L1 than the barriers cost (160 systems of 2k-28k cells: 62.8 ms
+  // without that limit, 62.8 with 5632, 52.4 with 4096, 55.1 with 3072; 200 of 2k-30k
+  // 83.5, 69.4, 72.8, 71.7; 304 of 2k-28k 91.4, 90.9, 94.0, 96.1).  Systems are laid out by
+  // their blocks and each group is one launch, side by side on its first system's second
+  // stream.
   constexpr long long kBlockCells = 1024, kMostCells = 4096;
   long long cells = 0;
   for (int k = 0; k < n; ++k) cells += ctxs[k]->N;

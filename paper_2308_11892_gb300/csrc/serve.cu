@@ -10,8 +10,8 @@
 // up, and their kernels overlap on the device.  A large request is then
 // solved by its slot.  A small one (at most batch_max_cells cells) is handed
 // to the batcher and its slot moves on: the batcher solves every small
-// request that is set up and waiting in one launch (cptr_solve_batch, one
-// thread block per system), while the next ones gather for the launch after
+// request that is set up and waiting in one call (cptr_solve_batch, one thread
+// block or cluster per system), while the next ones gather for the call after
 // it.  Each request owns its hierarchy and Krylov state until it finishes;
 // its result does not depend on what else runs (every reduction has a fixed
 // order, and a system's batched result is the same in any batch).

@@ -96,9 +96,9 @@ __global__ void k_qi_w(int N, const double* __restrict__ v, const int32_t* __res
 
 // Ahat_ij = A_ij[e,e] - W_i A_ij[h,e], scattered into the ne N scalar CSR whose
 // row ne i + r holds, for each block column j, the entries ne j .. ne j + ne - 1.
-// One warp per cell, a lane per entry: the lanes read whole blocks and write
-// consecutive entries, which the lines of
-// 128 bytes bound (200x200x100 grid: a thread per cell 2.9 ms, now 1.2).
+// One warp per cell, a lane per entry: bound by the 128-byte lines it touches, so the
+// lanes read whole blocks and write consecutive entries (200x200x100 grid: a thread
+// per cell 2.9 ms, now 1.2).
 __global__ void k_qi_ahat(int N, const int32_t* __restrict__ rp, const int32_t* __restrict__ ci,
                           const double* __restrict__ v, const double* __restrict__ W, int e0,
                           int e1, int h0, int h1, int h2, int32_t* __restrict__ Arp,
@@ -2052,7 +2052,7 @@ __device__ __forceinline__ void gj_push(V* local_ptr, unsigned rank, V v) {
 // integer pipes, every column of every slice is active, and no index is divided.
 // [M | I] beside each other and an FP64 compare per element took 1.40 ms at n = 208
 // and 0.68 at n = 146; in place with a fused update 0.80 and 0.44, which the separate
-// roundings lengthen by a fifth (64x64x32 grid's coarsest level 1.55 -> 1.87 ms).
+// roundings lengthen by a fifth (n = 245: 1.55 -> 1.87 ms).
 __global__ void __launch_bounds__(kGjThreads) k_gauss_jordan_cluster(int n, int w,
                                                                      const double* __restrict__ M,
                                                                      double* __restrict__ inv,
@@ -2197,8 +2197,9 @@ cptr_status acc_launch(cptr_ctx* c, void (*kern)(AccArgs, int, int), int rows_pe
   return CPTR_OK;
 }
 // Rows [from, ...) of class cls (about `rows` of them) with the class's kernel.
-// Short rows of B (at most six entries on average: interpolation operators) take
-// the lane-group kernels up to 256 columns, others a warp per row.
+// In the smallest class short rows of B (at most six entries on average: interpolation
+// operators) take the lane-group kernel; all others take a warp per row, the largest
+// class a block.
 cptr_status acc_run(cptr_ctx* c, AccArgs a, int cls, int from, int rows, bool short_b) {
   constexpr int W = kAccThreads / 32;
   switch (cls) {
@@ -2275,7 +2276,10 @@ cptr_status check_count_fits(cptr_ctx* c, const int32_t* cnt, int n, long long b
 // tables fit in kCap slots.
 cptr_status spgemm_fallback(cptr_ctx* c, const DCSR& A, const DCSR& B, DCSR& C);
 
-// Rows up to which a product is one launch: every warp of the GPU has one or two.
+// Rows up to which a product is one launch, of the class of its longest row: binning
+// would cost a launch and a read-back more than such a product takes.  (Up to 512
+// slots every warp of the GPU has one or two rows; the tables of the larger classes
+// leave fewer warps resident, up to seven rounds of them.)
 constexpr int kAccOneClass = 4096;
 
 // C = A * B in one pass: every row writes its sorted columns and sums into a slot

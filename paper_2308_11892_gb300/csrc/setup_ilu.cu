@@ -498,7 +498,7 @@ __global__ void k_sched_fill(int npos, const int32_t* __restrict__ ord,
   if (dinv) dinv[16 * (size_t)p + q] = (T)LU[16 * (size_t)diag[i] + q];
 }
 
-// level sets by repeated sweeps until a sweep changes nothing
+// Level sets of the rows in one pass (k_level_syncfree), and their number.
 cptr_status compute_levels(cptr_ctx* c, bool upper, int32_t* lvl, int* nlev) {
   int N = c->N;
   unsigned* ctr;
